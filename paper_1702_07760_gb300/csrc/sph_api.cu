@@ -117,6 +117,10 @@ struct sph_sim {
     unsigned long long *pair_tot = nullptr;
     double last_dt = 0.0;
     double *diag_out = nullptr, *diag_grav = nullptr;
+    DiagBlock *diag_blk = nullptr;        // the blocks of a diagnostics launch
+    double *diag_part = nullptr;          // their partial sums
+    unsigned *diag_arrived = nullptr;     // per instance, blocks done (reset by the last)
+    int diag_blocks = 0;
     double *read_buf = nullptr;
     int *read_ibuf = nullptr;
     int64_t step = 0;
@@ -959,6 +963,10 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
         s->own_stream = true;
     }
     const size_t N = (size_t)std::max<int64_t>(n, 1);
+    std::vector<DiagBlock> diag_blk;
+    for (int q = 0; q < k; ++q)
+        for (int64_t b = 0; b * DIAG_TILE < counts[q]; ++b) diag_blk.push_back({q, (int)b});
+    s->diag_blocks = (int)diag_blk.size();
     int err = 0;
     for (int b = 0; b < 2 && !err; ++b) {
         Dev &d = s->buf[b];
@@ -1008,6 +1016,9 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
         err |= s->alloc(&s->sort.perm, N);
         err |= s->alloc(&s->sort.tile_sums, (size_t)s->ntiles);
         err |= s->alloc(&s->diag_out, (size_t)k * DIAG_STRIDE);
+        err |= s->alloc(&s->diag_blk, diag_blk.size());
+        err |= s->alloc(&s->diag_part, diag_blk.size() * DIAG_SUMS);
+        err |= s->alloc(&s->diag_arrived, (size_t)k);
         err |= s->alloc(&s->diag_grav, 4);
         err |= s->alloc(&s->read_buf, N * 9 + 16);
         err |= s->alloc(&s->read_ibuf, N);
@@ -1074,6 +1085,11 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
     std::vector<long long> fl(s->first.begin(), s->first.end());
     if ((e = cudaMemcpyAsync(s->dfirst, fl.data(), sizeof(long long) * (k + 1), cudaMemcpyHostToDevice, st)) !=
         cudaSuccess)
+        return cuda_fail(e);
+    if ((e = cudaMemsetAsync(s->diag_out, 0, sizeof(double) * k * DIAG_STRIDE, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = cudaMemsetAsync(s->diag_arrived, 0, sizeof(unsigned) * k, st)) != cudaSuccess) return cuda_fail(e);
+    if (!diag_blk.empty() && (e = cudaMemcpyAsync(s->diag_blk, diag_blk.data(), sizeof(DiagBlock) * diag_blk.size(),
+                                                  cudaMemcpyHostToDevice, st)) != cudaSuccess)
         return cuda_fail(e);
     double grav[4] = {0, 0, 0, 0};
     for (int c = 0; c < dim; ++c) grav[c] = P0.g[c];
@@ -1885,21 +1901,16 @@ int sph_diag_instances(sph_handle s, double *out)
     const int k = s->ninst;
     for (int q = 0; q < 12 * k; ++q) out[q] = 0.0;
     if (s->n == 0) return SPH_OK;
-    const size_t n = (size_t)s->n, dim = (size_t)s->dim;
-    double *x = s->read_buf, *u = s->read_buf + n * dim;
-    // original-order positions (instance frames), velocities and tags
     if (s->dim == 2) {
-        k_unpermute<2><<<s->blocks(s->n), 256, 0, s->stream>>>(s->D(), RK_X, x, s->read_ibuf);
-        k_unpermute<2><<<s->blocks(s->n), 256, 0, s->stream>>>(s->D(), RK_U, u, s->read_ibuf);
-        k_unpermute<2><<<s->blocks(s->n), 256, 0, s->stream>>>(s->D(), RK_TAG, x, s->read_ibuf);
-        k_diag_inst<2><<<k, DIAG_THREADS, 0, s->stream>>>(s->dfirst, x, u, s->read_ibuf, s->dinst, s->diag_grav,
-                                                           s->diag_out);
+        k_diag_sums<2><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->D(), s->dfirst, s->diag_blk, s->diag_grav,
+                                                                       s->diag_part, s->diag_arrived, s->diag_out);
+        k_diag_cov<2><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->D(), s->dfirst, s->diag_blk, s->diag_part,
+                                                                      s->diag_arrived, s->diag_out);
     } else {
-        k_unpermute<3><<<s->blocks(s->n), 256, 0, s->stream>>>(s->D(), RK_X, x, s->read_ibuf);
-        k_unpermute<3><<<s->blocks(s->n), 256, 0, s->stream>>>(s->D(), RK_U, u, s->read_ibuf);
-        k_unpermute<3><<<s->blocks(s->n), 256, 0, s->stream>>>(s->D(), RK_TAG, x, s->read_ibuf);
-        k_diag_inst<3><<<k, DIAG_THREADS, 0, s->stream>>>(s->dfirst, x, u, s->read_ibuf, s->dinst, s->diag_grav,
-                                                           s->diag_out);
+        k_diag_sums<3><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->D(), s->dfirst, s->diag_blk, s->diag_grav,
+                                                                       s->diag_part, s->diag_arrived, s->diag_out);
+        k_diag_cov<3><<<s->diag_blocks, DIAG_THREADS, 0, s->stream>>>(s->D(), s->dfirst, s->diag_blk, s->diag_part,
+                                                                      s->diag_arrived, s->diag_out);
     }
     CU(cudaGetLastError());
     std::vector<double> r((size_t)k * DIAG_STRIDE);
