@@ -108,8 +108,8 @@ struct Surrogate {
     float *Z0, *h[3], *degs, *Z1[2], *Z2, *Y;
     float4 *NF;                  // per node: u / sd_edge_u (xyz), density deviation / sd_edge_rho
     // backward
-    float *dYf, *dZf, *dA, *dh, *dh2, *dS;
-    bf16 *dYb, *dZb, *dAb, *dhb, *dPQ, *T1, *T2;
+    float *dYf, *dZf, *dA, *dh, *dS;
+    bf16 *dYb, *dZb, *dAb, *dhb, *dPQ;
     double *loss_d = nullptr;
     unsigned *err = nullptr;
     // judge snapshots (original order)
@@ -152,21 +152,34 @@ __device__ __forceinline__ float dsilu(float z)
     return s * (1.f + z * (1.f - s));
 }
 
-// dst[(row_off + r) * ld + c] = W[r][c], or transposed dst[c * ld + row_off + r].
-__global__ void k_pack(const float *W, int rows, int cols, bf16 *dst, int ld, int row_off, int transpose)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= rows * cols) return;
-    const int r = k / cols, c = k % cols;
-    const bf16 v = __float2bfloat16_rn(W[k]);
-    if (transpose) dst[(size_t)c * ld + row_off + r] = v;
-    else dst[(size_t)(row_off + r) * ld + c] = v;
-}
+// The weights as the contractions read them, one launch for all tensors
+// (27 launches of 3 us each before): job y copies W (rows x cols of theta at
+// off) to BF16 dst[(row_off + r) * ld + c], transposed dst[c * ld + row_off +
+// r], or (FP32 vectors, biases) dstf[c].
+struct PackJob {
+    bf16 *dst;
+    float *dstf;
+    int off, rows, cols, ld, row_off, transpose;
+};
+constexpr int PACK_JOBS = 3 + 2 * 11 + 4 + 1;
+struct PackTable {
+    PackJob job[PACK_JOBS];
+};
 
-__global__ void k_copy_f(const float *src, float *dst, int count)
+__global__ void k_pack(const float *theta, const __grid_constant__ PackTable t)
 {
+    const PackJob &p = t.job[blockIdx.y];
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < count) dst[k] = src[k];
+    if (k >= p.rows * p.cols) return;
+    const int r = k / p.cols, c = k % p.cols;
+    const float w = theta[p.off + k];
+    if (p.dstf) {
+        p.dstf[k] = w;
+        return;
+    }
+    const bf16 v = __float2bfloat16_rn(w);
+    if (p.transpose) p.dst[(size_t)c * p.ld + p.row_off + r] = v;
+    else p.dst[(size_t)(p.row_off + r) * p.ld + c] = v;
 }
 
 // Normalised node inputs [u, (rho - rho0)/rho0, oil, wall, T a,
@@ -231,7 +244,10 @@ __device__ __forceinline__ bool edge_features(const Dev &d, const Grid &g, float
 // The pair-only part of the edge features: r_ij / 2h (DIM), |r_ij| / 2h,
 // phase_i != phase_j.  The state-difference channels of edge_features are
 // linear in node quantities, so the forward pass folds them into the node
-// terms (k_pq_fold) and the edge phase needs only these.
+// terms (the epilogue of the P, Q layer: with f_i the node's scaled (u, delta)
+// channels and W3d their columns of W3, W3d (f_i - f_j) = W3d f_i - W3d f_j, so
+// P'_i = P_i + W3d f_i and Q'_j = Q_j - W3d f_j give the same pre-activation
+// P'_i + Q'_j + W3g e_ij) and the edge phase needs only these.
 template <int DIM>
 __device__ __forceinline__ bool edge_geom(const Dev &d, const Grid &g, float R2, float inv2h, const float4 &oi,
                                           int phi, unsigned e, int &j, float (&ef)[DIM + 2])
@@ -344,41 +360,6 @@ __device__ __forceinline__ unsigned stage_geom_h2(const Dev &d, const Grid &g, f
     return mask;
 }
 
-// Folds the state-difference channels of the first edge layer into the node
-// terms: with f_i the node's scaled (u, delta) channels and W3d their columns
-// of W3, W3d (f_i - f_j) = W3d f_i - W3d f_j, so P'_i = P_i + W3d f_i and
-// Q'_j = Q_j - W3d f_j give the same pre-activation P'_i + Q'_j + W3g e_ij.
-// One thread per node and four features; FP32 sums, FP16 results.
-template <int DIM>
-__global__ void __launch_bounds__(256) k_pq_fold(int n, const float4 *NF, const __half *PQ, const float *W3,
-                                                 __half *PQf)
-{
-    constexpr int NE = 2 * DIM + 3;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int i = (int)(t >> 5);
-    if (i >= n) return;
-    const int f0 = (int)(t & 31) * 4;
-    const float4 f = NF[i];
-    const float fa[3] = {f.x, f.y, f.z};
-    float pv[4], qv[4];
-    load4(PQ + (size_t)i * 2 * H + f0, pv);
-    load4(PQ + (size_t)i * 2 * H + H + f0, qv);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float *w = W3 + (size_t)(f0 + q) * NE;
-        float sdiff = w[2 * DIM + 2] * f.w;
-#pragma unroll
-        for (int a = 0; a < DIM; ++a) sdiff = fmaf(w[DIM + 2 + a], fa[a], sdiff);
-        pv[q] += sdiff;
-        qv[q] -= sdiff;
-    }
-    __half2 *pp = (__half2 *)(PQf + (size_t)i * 2 * H + f0), *qq = (__half2 *)(PQf + (size_t)i * 2 * H + H + f0);
-    pp[0] = __floats2half2_rn(pv[0], pv[1]);
-    pp[1] = __floats2half2_rn(pv[2], pv[3]);
-    qq[0] = __floats2half2_rn(qv[0], qv[1]);
-    qq[1] = __floats2half2_rn(qv[2], qv[3]);
-}
-
 __device__ __forceinline__ __half2 tanh_h2(__half2 x)
 {
     uint32_t r;
@@ -388,7 +369,7 @@ __device__ __forceinline__ __half2 tanh_h2(__half2 x)
 
 // Forward edge phase: one warp per receiver i, four features per lane.
 // S_i = (1/k_ref) sum_j SiLU(P'_i + Q'_j + W3g e_ij) over list entries with
-// |r_ij| < 2h (the folded node terms of k_pq_fold and the pair features);
+// |r_ij| < 2h (the folded node terms and the pair features);
 // degs_i = deg_i / k_ref.  Entries are decoded 32 at a time,
 // one per lane; the sender rows Q_j of every valid entry of the batch are
 // then copied to shared memory with cp.async (all in flight together).  The
@@ -600,30 +581,6 @@ __global__ void k_colsum(const float *src, int ld, int cols, int n, const float 
     if (s != 0.f) atomicAdd(dst + c, s);
 }
 
-// dst[c][r] = src[r][c] for r < rows (rows padded up to a multiple of 32), c < cols.
-__global__ void k_transpose(const bf16 *src, int ld_src, int rows, int cols, bf16 *dst, int ld_dst)
-{
-    __shared__ bf16 tile[32][33];
-    const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int r = r0 + k, c = c0 + threadIdx.x;
-        tile[k][threadIdx.x] = (r < rows && c < cols) ? src[(size_t)r * ld_src + c] : __float2bfloat16_rn(0.f);
-    }
-    __syncthreads();
-    for (int k = threadIdx.y; k < 32; k += blockDim.y) {
-        const int c = c0 + k, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) dst[(size_t)c * ld_dst + r] = tile[threadIdx.x][k];
-    }
-}
-
-__global__ void k_add(const float *a, int lda, const float *b, int ldb, float *out, int ldo, int rows, int cols)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= rows * cols) return;
-    const int r = k / cols, c = k % cols;
-    out[(size_t)r * ldo + c] = a[(size_t)r * lda + c] + b[(size_t)r * ldb + c];
-}
-
 // Targets from the state after k plain steps (original order, instance
 // frame) against the current state (sorted), masked squared error, dL/dy.
 template <int DIM>
@@ -760,13 +717,17 @@ struct Epi {
     int ldz = 0;
     const float *residual = nullptr;
     int ldr = 0;
+    const float *residual2 = nullptr;
+    int ldr2 = 0;
     int act = 0;
     const float *dact = nullptr;
     int lddact = 0;
-    int atomic = 0;
-    int k_split = 0;
-    int n_store = 0;
     int cb_half = 0;
+    // the P, Q layer: folded node terms (see umma::GemmArgs)
+    const float4 *fold_f = nullptr;
+    const float *fold_w = nullptr;
+    int dim = 0;
+    __half *fold_out = nullptr;
 };
 
 int mm(Surrogate &S, cudaStream_t st, const bf16 *A, int lda, const bf16 *B, int ldb, int M, int N, int K,
@@ -780,7 +741,7 @@ int mm(Surrogate &S, cudaStream_t st, const bf16 *A, int lda, const bf16 *B, int
     g.M = M;
     g.N = N;
     g.K = K;
-    g.k_split = e.k_split > 0 ? e.k_split : ((K + umma::BK - 1) / umma::BK) * umma::BK;
+    g.k_split = ((K + umma::BK - 1) / umma::BK) * umma::BK;
     g.Cf = e.Cf;
     g.ldcf = e.ldcf;
     g.Cb = e.Cb;
@@ -792,46 +753,50 @@ int mm(Surrogate &S, cudaStream_t st, const bf16 *A, int lda, const bf16 *B, int
     g.ldz = e.ldz;
     g.residual = e.residual;
     g.ldr = e.ldr;
+    g.residual2 = e.residual2;
+    g.ldr2 = e.ldr2;
     g.act = e.act;
     g.dact = e.dact;
     g.lddact = e.lddact;
-    g.atomic = e.atomic;
-    g.n_store = e.n_store;
     g.cb_half = e.cb_half;
     g.err = S.err;
-    cudaError_t err = umma::gemm(g, st);
+    if (e.fold_out) {
+        g.fold_f = e.fold_f;
+        g.fold_w = e.fold_w;
+        g.fold_ldw = 2 * e.dim + 3;
+        g.fold_v = e.dim + 2;
+        g.fold_s = 2 * e.dim + 2;
+        g.fold_dim = e.dim;
+        g.fold_out = e.fold_out;
+        g.fold_ld = N;
+    }
+    // every layer of the network has a shape of k_layer, whose epilogue alone folds and adds two residuals
+    cudaError_t err = umma::layer_fits(g) ? umma::layer(g, st) : cudaErrorInvalidValue;
     if (err != cudaSuccess) return set_error(SPH_ECUDA, std::string("gemm: ") + cudaGetErrorString(err));
     return SPH_OK;
 }
 
-// dW (rows x cols, ld cols, in the flat gradient) += dY^T X, with dY^T (rows x npad) and X^T (cols x npad).
-int mm_wgrad(Surrogate &S, cudaStream_t st, const bf16 *dYT, int rows, const bf16 *XT, int cols, float *dW,
-             int n_store = 0)
+// dW (rows x cols, ld cols, in the flat gradient) += dY^T X over the nodes: dY with fy
+// features (the first `rows` of them, or with dW2 both halves of 256), X with fx.  4096
+// nodes a block.
+int wgrad(Surrogate &S, cudaStream_t st, const bf16 *dY, int ldy, int fy, const bf16 *X, int ldx, int fx, float *dW,
+          int rows, int cols, float *dW2 = nullptr)
 {
-    Epi e;
-    e.Cf = dW;
-    e.ldcf = n_store > 0 ? n_store : cols;
-    e.atomic = 1;
-    e.n_store = n_store;
-    e.k_split = 4096;
-    return mm(S, st, dYT, S.npad, XT, S.npad, rows, cols, S.npad, e);
-}
-
-int transpose(Surrogate &S, cudaStream_t st, const bf16 *src, int ld, int cols, bf16 *dst)
-{
-    dim3 grid(S.npad / 32, (cols + 31) / 32);
-    k_transpose<<<grid, dim3(32, 8), 0, st>>>(src, ld, S.npad, cols, dst, S.npad);
-    CUR(cudaGetLastError());
+    cudaError_t err = umma::wgrad(dY, ldy, fy, X, ldx, fx, S.n, dW, dW2, cols, rows, cols, 4096, S.err, st);
+    if (err != cudaSuccess) return set_error(SPH_ECUDA, std::string("wgrad: ") + cudaGetErrorString(err));
     return SPH_OK;
 }
 
 int pack_weights(Surrogate &S, cudaStream_t st)
 {
     const Layout &L = S.L;
-    const float *T = S.theta;
+    PackTable t{};
+    int jobs = 0, most = 0;
     auto pk = [&](int off, int rows, int cols, bf16 *dst, int ld, int row_off, int tr) {
-        k_pack<<<nb(rows * cols), 256, 0, st>>>(T + off, rows, cols, dst, ld, row_off, tr);
+        t.job[jobs++] = {dst, nullptr, off, rows, cols, ld, row_off, tr};
+        most = std::max(most, rows * cols);
     };
+    auto copy = [&](int off, int count, float *dst) { t.job[jobs++] = {nullptr, dst, off, 1, count, 0, 0, 0}; };
     pk(L.enc1w, H, L.nin, S.Wenc1, FIN, 0, 0);
     pk(L.enc2w, H, H, S.Wenc2, H, 0, 0);
     pk(L.enc2w, H, H, S.Wenc2T, H, 0, 1);
@@ -846,13 +811,14 @@ int pack_weights(Surrogate &S, cudaStream_t st)
         pk(L.n1[r], H, 2 * H, S.Wn1T[r], H, 0, 1);
         pk(L.n2[r], H, H, S.Wn2[r], H, 0, 0);
         pk(L.n2[r], H, H, S.Wn2T[r], H, 0, 1);
-        k_copy_f<<<1, H, 0, st>>>(T + L.b1[r], S.bpq[r], H);
+        copy(L.b1[r], H, S.bpq[r]);
     }
     pk(L.dec1w, H, H, S.Wd1, H, 0, 0);
     pk(L.dec1w, H, H, S.Wd1T, H, 0, 1);
     pk(L.dec2w, L.nout, H, S.Wd2, H, 0, 0);
     pk(L.dec2w, L.nout, H, S.Wd2T, FOUT, 0, 1);
-    k_copy_f<<<1, 32, 0, st>>>(T + L.dec2b, S.bd2, L.nout);
+    copy(L.dec2b, L.nout, S.bd2);
+    k_pack<<<dim3(nb(most), jobs), 256, 0, st>>>(S.theta, t);
     CUR(cudaGetLastError());
     return SPH_OK;
 }
@@ -921,12 +887,9 @@ int alloc_backward(Surrogate &S)
     e |= dalloc(S, &S.dA, P * 2 * H);
     e |= dalloc(S, &S.dAb, P * 2 * H);
     e |= dalloc(S, &S.dh, P * H);
-    e |= dalloc(S, &S.dh2, P * H);
     e |= dalloc(S, &S.dhb, P * H);
     e |= dalloc(S, &S.dS, P * H);
     e |= dalloc(S, &S.dPQ, P * 2 * H);
-    e |= dalloc(S, &S.T1, P * 2 * H);
-    e |= dalloc(S, &S.T2, P * 2 * H);
     if (e) return SPH_ENOMEM;
     CUR(cudaDeviceSynchronize());
     return SPH_OK;
@@ -970,20 +933,22 @@ int forward(Surrogate &S, const SimView &v, bool training)
         {
             Epi e;
             e.bias = S.bpq[r];
-            e.Cb = (bf16 *)S.PQ[r];
+            // the backward pass reads the unfolded terms
+            e.Cb = training ? (bf16 *)S.PQ[r] : nullptr;
             e.cb_half = 1;
             e.ldcb = 2 * H;
+            e.fold_f = S.NF;
+            e.fold_w = T + L.w3[r];
+            e.dim = v.dim;
+            e.fold_out = S.PQf;
             if ((rc = mm(S, st, S.A1[r], 2 * H, S.Wpq[r], H, n, 2 * H, H, e))) return rc;
         }
-        if (v.dim == 2) {
-            k_pq_fold<2><<<nb(n * 32, 256), 256, 0, st>>>(n, S.NF, S.PQ[r], T + L.w3[r], S.PQf);
+        if (v.dim == 2)
             k_edge_fwd<2><<<nb(n * 32, EWF), EWF, 0, st>>>(v.d, v.g, R2, inv2h, S.PQf, T + L.w3[r], invk, S.S[r],
                                                            S.degs);
-        } else {
-            k_pq_fold<3><<<nb(n * 32, 256), 256, 0, st>>>(n, S.NF, S.PQ[r], T + L.w3[r], S.PQf);
+        else
             k_edge_fwd<3><<<nb(n * 32, EWF), EWF, 0, st>>>(v.d, v.g, R2, inv2h, S.PQf, T + L.w3[r], invk, S.S[r],
                                                            S.degs);
-        }
         CUR(cudaGetLastError());
         {
             Epi e;
@@ -1047,9 +1012,7 @@ int backward(Surrogate &S, const SimView &v)
     int rc = 0;
     CUR(cudaMemsetAsync(G, 0, sizeof(float) * L.total, st));
     // decoder, layer 2
-    if ((rc = transpose(S, st, S.dYb, FOUT, FOUT, S.T1))) return rc;
-    if ((rc = transpose(S, st, S.A2, H, H, S.T2))) return rc;
-    if ((rc = mm_wgrad(S, st, S.T1, L.nout, S.T2, H, G + L.dec2w))) return rc;
+    if ((rc = wgrad(S, st, S.dYb, FOUT, FOUT, S.A2, H, H, G + L.dec2w, L.nout, H))) return rc;
     k_colsum<<<cs_blocks, 256, 0, st>>>(S.dYf, FOUT, L.nout, n, nullptr, G + L.dec2b);
     {
         Epi e;
@@ -1063,9 +1026,7 @@ int backward(Surrogate &S, const SimView &v)
         if ((rc = mm(S, st, S.dYb, FOUT, S.Wd2T, FOUT, n, H, FOUT, e))) return rc;
     }
     // decoder, layer 1
-    if ((rc = transpose(S, st, S.dZb, H, H, S.T1))) return rc;
-    if ((rc = transpose(S, st, S.hLb, H, H, S.T2))) return rc;
-    if ((rc = mm_wgrad(S, st, S.T1, H, S.T2, H, G + L.dec1w))) return rc;
+    if ((rc = wgrad(S, st, S.dZb, H, H, S.hLb, H, H, G + L.dec1w, H, H))) return rc;
     k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, G + L.dec1b);
     {
         Epi e;
@@ -1079,9 +1040,7 @@ int backward(Surrogate &S, const SimView &v)
     for (int r = 1; r >= 0; --r) {
         const bf16 *hb = r == 0 ? S.A1[0] : S.A1[1];   // h_r in BF16: left half of [h, M]
         // node MLP, layer 2 (residual: dh passes through)
-        if ((rc = transpose(S, st, S.dhb, H, H, S.T1))) return rc;
-        if ((rc = transpose(S, st, S.G1[r], H, H, S.T2))) return rc;
-        if ((rc = mm_wgrad(S, st, S.T1, H, S.T2, H, G + L.n2[r]))) return rc;
+        if ((rc = wgrad(S, st, S.dhb, H, H, S.G1[r], H, H, G + L.n2[r], H, H))) return rc;
         k_colsum<<<cs_blocks, 256, 0, st>>>(S.dh, H, H, n, nullptr, G + L.n2b[r]);
         {
             Epi e;
@@ -1095,9 +1054,7 @@ int backward(Surrogate &S, const SimView &v)
             if ((rc = mm(S, st, S.dhb, H, S.Wn2T[r], H, n, H, H, e))) return rc;
         }
         // node MLP, layer 1 on [h, M]
-        if ((rc = transpose(S, st, S.dZb, H, H, S.T1))) return rc;
-        if ((rc = transpose(S, st, S.A1[r], 2 * H, 2 * H, S.T2))) return rc;
-        if ((rc = mm_wgrad(S, st, S.T1, H, S.T2, 2 * H, G + L.n1[r]))) return rc;
+        if ((rc = wgrad(S, st, S.dZb, H, H, S.A1[r], 2 * H, 2 * H, G + L.n1[r], H, 2 * H))) return rc;
         k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, G + L.n1b[r]);
         {
             Epi e;
@@ -1108,9 +1065,7 @@ int backward(Surrogate &S, const SimView &v)
             if ((rc = mm(S, st, S.dZb, H, S.Wn1T[r], H, n, 2 * H, H, e))) return rc;
         }
         // second edge layer, applied after the sum: M = S We2^T + degs be2
-        if ((rc = transpose(S, st, S.dAb + H, 2 * H, H, S.T1))) return rc;
-        if ((rc = transpose(S, st, S.S[r], H, H, S.T2))) return rc;
-        if ((rc = mm_wgrad(S, st, S.T1, H, S.T2, H, G + L.we2[r]))) return rc;
+        if ((rc = wgrad(S, st, S.dAb + H, 2 * H, H, S.S[r], H, H, G + L.we2[r], H, H))) return rc;
         k_colsum<<<cs_blocks, 256, 0, st>>>(S.dA + H, 2 * H, H, n, S.degs, G + L.be2[r]);
         {
             Epi e;
@@ -1127,16 +1082,14 @@ int backward(Surrogate &S, const SimView &v)
                                                          S.dS, S.dPQ, G + L.w3[r], G + L.b1[r]);
         CUR(cudaGetLastError());
         // first edge layer, node parts: P = h W1^T + b1, Q = h W2^T
-        if ((rc = transpose(S, st, S.dPQ, 2 * H, 2 * H, S.T1))) return rc;
-        if ((rc = transpose(S, st, hb, 2 * H, H, S.T2))) return rc;
-        if ((rc = mm_wgrad(S, st, S.T1, H, S.T2, H, G + L.w1[r]))) return rc;
-        if ((rc = mm_wgrad(S, st, S.T1 + (size_t)H * S.npad, H, S.T2, H, G + L.w2[r]))) return rc;
+        if ((rc = wgrad(S, st, S.dPQ, 2 * H, 2 * H, hb, 2 * H, H, G + L.w1[r], H, H, G + L.w2[r]))) return rc;
         // dh_r = dh_{r+1} + d[h part of n1 input] + dP W1 + dQ W2
-        k_add<<<nb(n * H), 256, 0, st>>>(S.dh, H, S.dA, 2 * H, S.dh2, H, n, H);
         {
             Epi e;
-            e.residual = S.dh2;
+            e.residual = S.dh;   // in place: a row's elements are read before they are written
             e.ldr = H;
+            e.residual2 = S.dA;
+            e.ldr2 = 2 * H;
             e.Cf = S.dh;
             e.ldcf = H;
             e.Cb = S.dhb;
@@ -1145,9 +1098,7 @@ int backward(Surrogate &S, const SimView &v)
         }
     }
     // encoder, layer 2
-    if ((rc = transpose(S, st, S.dhb, H, H, S.T1))) return rc;
-    if ((rc = transpose(S, st, S.A0, H, H, S.T2))) return rc;
-    if ((rc = mm_wgrad(S, st, S.T1, H, S.T2, H, G + L.enc2w))) return rc;
+    if ((rc = wgrad(S, st, S.dhb, H, H, S.A0, H, H, G + L.enc2w, H, H))) return rc;
     k_colsum<<<cs_blocks, 256, 0, st>>>(S.dh, H, H, n, nullptr, G + L.enc2b);
     {
         Epi e;
@@ -1161,9 +1112,7 @@ int backward(Surrogate &S, const SimView &v)
         if ((rc = mm(S, st, S.dhb, H, S.Wenc2T, H, n, H, H, e))) return rc;
     }
     // encoder, layer 1
-    if ((rc = transpose(S, st, S.dZb, H, H, S.T1))) return rc;
-    if ((rc = transpose(S, st, S.X16, FIN, FIN, S.T2))) return rc;
-    if ((rc = mm_wgrad(S, st, S.T1, H, S.T2, FIN, G + L.enc1w, L.nin))) return rc;
+    if ((rc = wgrad(S, st, S.dZb, H, H, S.X16, FIN, FIN, G + L.enc1w, H, L.nin))) return rc;
     k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, G + L.enc1b);
     CUR(cudaGetLastError());
     return SPH_OK;
