@@ -89,7 +89,7 @@ Layout make_layout(int dim)
 }
 
 struct Surrogate {
-    int dim = 0, n = 0, npad = 0;
+    int dim = 0, n = 0, npad = 0, sms = 0;
     Layout L;
     float k_ref = 1.f, t_jump = 0.f, sd_edge_u = 1.f, sd_edge_rho = 1.f;
     double t_jump64 = 0.0;       // the jump's time span (the device clock advances by it)
@@ -320,46 +320,6 @@ __device__ __forceinline__ unsigned stage_entries(const Dev &d, const Grid &g, f
     return mask;
 }
 
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
-                 "l"(gmem)
-                 : "memory");
-}
-
-// Slots of the forward edge phase: the DIM + 2 pair features and the sender.
-template <int DIM>
-__host__ __device__ constexpr int geom_slot_width() { return ((DIM + 3) + 3) / 4 * 4; }
-
-// Lane-parallel decoding of up to 32 entries for the forward edge phase: the
-// pair features as duplicated FP16 pairs and the sender index after them.
-template <int DIM>
-__device__ __forceinline__ unsigned stage_geom_h2(const Dev &d, const Grid &g, float R2, float inv2h,
-                                                  const float4 &oi, int phi, int i, int k0, int cnt,
-                                                  uint32_t (*slot)[geom_slot_width<DIM>()])
-{
-    constexpr int NG = DIM + 2;
-    const int lane = threadIdx.x & 31;
-    const int k = k0 + lane;
-    bool valid = false;
-    if (k < cnt) {
-        int j;
-        float ef[NG];
-        valid = edge_geom<DIM>(d, g, R2, inv2h, oi, phi, d.nbr[(size_t)k * d.n + i], j, ef);
-        if (valid) {
-#pragma unroll
-            for (int c = 0; c < NG; ++c) {
-                const __half2 e2 = __float2half2_rn(ef[c]);
-                slot[lane][c] = *(const uint32_t *)&e2;
-            }
-            slot[lane][NG] = (uint32_t)j;
-        }
-    }
-    const unsigned mask = __ballot_sync(0xffffffffu, valid);
-    __syncwarp();
-    return mask;
-}
-
 __device__ __forceinline__ __half2 tanh_h2(__half2 x)
 {
     uint32_t r;
@@ -367,92 +327,164 @@ __device__ __forceinline__ __half2 tanh_h2(__half2 x)
     return *(const __half2 *)&r;
 }
 
-// Forward edge phase: one warp per receiver i, four features per lane.
+// Forward edge phase: half a warp per receiver i, eight features per lane.
 // S_i = (1/k_ref) sum_j SiLU(P'_i + Q'_j + W3g e_ij) over list entries with
-// |r_ij| < 2h (the folded node terms and the pair features);
-// degs_i = deg_i / k_ref.  Entries are decoded 32 at a time,
-// one per lane; the sender rows Q_j of every valid entry of the batch are
-// then copied to shared memory with cp.async (all in flight together).  The
-// pre-activation and SiLU run on feature pairs in FP16 (packed FMA, and
-// SiLU(z) = h + h tanh(h) with h = z/2); each batch's sum is added to an
-// FP32 accumulator.
-constexpr int EWF = 128;   // threads of the forward edge kernel (4 warps, one node each)
+// |r_ij| < 2h (the folded node terms and the pair features); degs_i = deg_i /
+// k_ref.  The pre-activation and SiLU run on feature pairs in FP16 (packed FMA,
+// and SiLU(z) = h + h tanh(h) with h = z/2); the sum of each 32 list entries is
+// added to an FP32 accumulator.
+//
+// Bound by instruction issue and the tanh unit (DRAM a few per cent): per edge
+// and 64 feature pairs, 10 packed operations a pair.  What is done per edge and
+// not per feature (the slot and sender-row reads, addresses, the loop) is
+// shared by a warp's two receivers and its eight features a lane: 58 warp
+// instructions an edge with a warp per receiver and four features a lane, about
+// 28 so.  The two receivers' next 32 entries are decoded lane-parallel (their
+// list columns are adjacent words) into 16-byte slots, the valid ones
+// compacted in list order: the pair features and a mask in FP16 (packed
+// arithmetic takes either half of a register as both) and the sender.  The
+// shorter of the two is padded with its last valid slot at mask 0 (a term that
+// is finite whenever the sum is), so the warp runs one uniform loop; sender rows
+// come straight from L1/L2, EDGE_U edges' loads issued before the first is
+// used.  Blocks are persistent: W3 stays in registers.
+// 656 600 particles, one round (GB300, profiler): 3.60 -> 2.40 ms; on 193 496,
+// 1.05 -> 0.69 ms with 463 M warp instructions instead of 762 M, the FP16 half of
+// the FMA pipe 65 % busy.  Five blocks an SM (96 registers) and four edges in
+// flight measured best (jump 6.7 ms; six blocks 7.5, eight 7.3, eight edges 6.8).
+#ifndef EDGE_U
+#define EDGE_U 4
+#endif
+#ifndef EDGE_BLOCKS
+#define EDGE_BLOCKS 5
+#endif
+constexpr int EWF = 128;   // threads of the forward edge kernel (4 warps, two receivers each)
 
 template <int DIM>
-__global__ void __launch_bounds__(EWF, 4) k_edge_fwd(Dev d, Grid g, float R2, float inv2h, const __half *PQ,
-                                                   const float *W3, float inv_kref, bf16 *S, float *degs)
+__global__ void __launch_bounds__(EWF, EDGE_BLOCKS)
+    k_edge_fwd(Dev d, Grid g, float R2, float inv2h, const __half *__restrict__ PQ, const float *W3, float inv_kref,
+               bf16 *S, float *degs)
 {
     constexpr int NE = 2 * DIM + 3;   // columns of W3 (the pair features are its first NG)
     constexpr int NG = DIM + 2;
-    constexpr int SWD = geom_slot_width<DIM>();
-    __shared__ __align__(16) uint32_t slots[EWF / 32][32][SWD];
-    __shared__ __align__(16) uint2 qrows[EWF / 32][32][32];   // [warp][entry][lane]: 4 FP16 features
-    const int wid = threadIdx.x >> 5;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (i >= d.n) return;
-    const int f0 = lane * 4;
-    __half2 w2[NG][2];   // W3 column c for features (f0, f0+1) and (f0+2, f0+3)
+    constexpr int U = EDGE_U;
+    constexpr int CAP = (32 + U - 1) / U * U;
+    __shared__ __align__(16) uint4 slots[EWF / 32][2][CAP];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int half = lane >> 4, f0 = (lane & 15) * 8;
+    __half2 w2[NG][4];   // W3 column c for the features (f0, f0 + 1), ...
 #pragma unroll
-    for (int c = 0; c < NG; ++c) {
-        w2[c][0] = __floats2half2_rn(W3[f0 * NE + c], W3[(f0 + 1) * NE + c]);
-        w2[c][1] = __floats2half2_rn(W3[(f0 + 2) * NE + c], W3[(f0 + 3) * NE + c]);
-    }
-    const uint2 praw = *(const uint2 *)(PQ + (size_t)i * 2 * H + f0);
-    const __half2 P0 = *(const __half2 *)&praw.x, P1 = *(const __half2 *)&praw.y;
+    for (int c = 0; c < NG; ++c)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            w2[c][q] = __floats2half2_rn(W3[(f0 + 2 * q) * NE + c], W3[(f0 + 2 * q + 1) * NE + c]);
     const __half2 half2c = __float2half2_rn(0.5f);
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    int deg = 0;
-    const float4 oi = d.pos[i];
-    const int phi = rec_phase(oi.w);
-    const int cnt = d.ncnt[i];
-    uint32_t(*slot)[SWD] = slots[wid];
-    uint2(*qr)[32] = qrows[wid];
-    for (int k0 = 0; k0 < cnt; k0 += 32) {
-        const unsigned valid = stage_geom_h2<DIM>(d, g, R2, inv2h, oi, phi, i, k0, cnt, slot);
-        deg += __popc(valid);
-        for (unsigned m = valid; m; m &= m - 1) {
-            const int sl = __ffs(m) - 1;
-            cp_async8(&qr[sl][lane], PQ + (size_t)slot[sl][NG] * 2 * H + H + f0);
-        }
-        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
-        __syncwarp();
-        __half2 s0 = __float2half2_rn(0.f), s1 = s0;
-        for (unsigned m = valid; m; m &= m - 1) {
-            const int sl = __ffs(m) - 1;
-            const uint2 raw = qr[sl][lane];
-            __half2 z0 = __hadd2(P0, *(const __half2 *)&raw.x);
-            __half2 z1 = __hadd2(P1, *(const __half2 *)&raw.y);
-            uint32_t e[SWD];
+    uint4(*const slot)[CAP] = slots[wid];
+    const uint4 *const mine = slot[half];
+    const __half *const Q = PQ + H + f0;
+    const int n = d.n;
+    const int stride = gridDim.x * (EWF / 32) * 2;
+    for (int base = (blockIdx.x * (EWF / 32) + wid) * 2; base < n; base += stride) {
+        // decoding: lane l takes receiver base + (l & 1) and entry l >> 1 of 16
+        const int di = min(base + (lane & 1), n - 1);
+        const float4 oi = d.pos[di];
+        const int phi = rec_phase(oi.w);
+        const int dcnt = base + (lane & 1) < n ? d.ncnt[di] : 0;
+        const int most = max(dcnt, __shfl_xor_sync(0xffffffffu, dcnt, 1));
+        // summing: this half's receiver
+        const int i = min(base + half, n - 1);
+        const uint4 praw = *(const uint4 *)(PQ + (size_t)i * 2 * H + f0);
+        const __half2 P[4] = {*(const __half2 *)&praw.x, *(const __half2 *)&praw.y, *(const __half2 *)&praw.z,
+                              *(const __half2 *)&praw.w};
+        float acc[8];
 #pragma unroll
-            for (int v4 = 0; v4 < SWD / 4; ++v4) {
-                const uint4 t4 = *(const uint4 *)&slot[sl][4 * v4];
-                e[4 * v4] = t4.x;
-                e[4 * v4 + 1] = t4.y;
-                e[4 * v4 + 2] = t4.z;
-                e[4 * v4 + 3] = t4.w;
-            }
+        for (int q = 0; q < 8; ++q) acc[q] = 0.f;
+        int deg = 0;
+        for (int k0 = 0; k0 < most; k0 += 32) {
+            int have0 = 0, have1 = 0;
+            __syncwarp();
 #pragma unroll
-            for (int c = 0; c < NG; ++c) {
-                const __half2 ec = *(const __half2 *)&e[c];
-                z0 = __hfma2(w2[c][0], ec, z0);
-                z1 = __hfma2(w2[c][1], ec, z1);
+            for (int pass = 0; pass < 2; ++pass) {
+                const int k = k0 + pass * 16 + (lane >> 1);
+                bool valid = false;
+                int j = 0;
+                float ef[NG];
+                if (k < dcnt)
+                    valid = edge_geom<DIM>(d, g, R2, inv2h, oi, phi, d.nbr[(size_t)k * n + di], j, ef);
+                const unsigned m = __ballot_sync(0xffffffffu, valid);
+                if (valid) {
+                    const unsigned own = m & (0x55555555u << (lane & 1));
+                    const __half2 a = __floats2half2_rn(ef[0], ef[1]), b = __floats2half2_rn(ef[2], ef[3]);
+                    const __half2 c = __floats2half2_rn(ef[NG - 1], 1.f);   // (2-D: the first half is not used)
+                    slot[lane & 1][((lane & 1) ? have1 : have0) + __popc(own & ((1u << lane) - 1u))] =
+                        make_uint4(*(const uint32_t *)&a, *(const uint32_t *)&b, *(const uint32_t *)&c, (uint32_t)j);
+                }
+                have0 += __popc(m & 0x55555555u);
+                have1 += __popc(m & 0xaaaaaaaau);
             }
-            const __half2 h0 = __hmul2(z0, half2c), h1 = __hmul2(z1, half2c);
-            s0 = __hadd2(s0, __hfma2(h0, tanh_h2(h0), h0));
-            s1 = __hadd2(s1, __hfma2(h1, tanh_h2(h1), h1));
+            __syncwarp();
+            const int cnt = half ? have1 : have0;
+            const int full = (max(have0, have1) + U - 1) / U * U;
+            // padding: the last valid slot (or, with none, the receiver itself) at mask 0
+            if (cnt < full) {
+                uint4 pad = make_uint4(0u, 0u, 0u, (uint32_t)i);
+                if (cnt > 0) {
+                    pad = mine[cnt - 1];
+                    pad.z &= 0xffffu;
+                }
+                for (int q = cnt + (lane & 15); q < full; q += 16) slot[half][q] = pad;
+            }
+            __syncwarp();
+            deg += cnt;
+            __half2 s[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] = __float2half2_rn(0.f);
+            for (int e0 = 0; e0 < full; e0 += U) {
+                uint4 sl[U], row[U];
+#pragma unroll
+                for (int t = 0; t < U; ++t) sl[t] = mine[e0 + t];
+#pragma unroll
+                for (int t = 0; t < U; ++t) row[t] = *(const uint4 *)(Q + (size_t)sl[t].w * (2 * H));
+#pragma unroll
+                for (int t = 0; t < U; ++t) {
+                    const __half2 q2[4] = {*(const __half2 *)&row[t].x, *(const __half2 *)&row[t].y,
+                                           *(const __half2 *)&row[t].z, *(const __half2 *)&row[t].w};
+                    const __half2 eab = *(const __half2 *)&sl[t].x, ecd = *(const __half2 *)&sl[t].y;
+                    const __half2 eem = *(const __half2 *)&sl[t].z;
+                    const __half2 ec[5] = {__low2half2(eab), __high2half2(eab), __low2half2(ecd), __high2half2(ecd),
+                                           __low2half2(eem)};
+                    const __half2 mask = __high2half2(eem);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        __half2 z = __hadd2(P[q], q2[q]);
+#pragma unroll
+                        for (int c = 0; c < NG; ++c) z = __hfma2(w2[c][q], ec[c], z);
+                        const __half2 h = __hmul2(z, half2c);
+                        // mask 1: the rounded sum s + x; mask 0: s
+                        s[q] = __hfma2(__hfma2(h, tanh_h2(h), h), mask, s[q]);
+                    }
+                }
+            }
+            if (cnt > 0)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float2 a = __half22float2(s[q]);
+                    acc[2 * q] += a.x;
+                    acc[2 * q + 1] += a.y;
+                }
         }
-        const float2 a0 = __half22float2(s0), a1 = __half22float2(s1);
-        acc[0] += a0.x;
-        acc[1] += a0.y;
-        acc[2] += a1.x;
-        acc[3] += a1.y;
-        __syncwarp();
+        if (base + half < n) {
+            uint4 o;
+            uint32_t ow[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const __nv_bfloat162 v = __floats2bfloat162_rn(acc[2 * q] * inv_kref, acc[2 * q + 1] * inv_kref);
+                ow[q] = *(const uint32_t *)&v;
+            }
+            o = make_uint4(ow[0], ow[1], ow[2], ow[3]);
+            *(uint4 *)(S + (size_t)i * H + f0) = o;
+            if ((lane & 15) == 0) degs[i] = deg * inv_kref;
+        }
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[q] *= inv_kref;
-    store4(S + (size_t)i * H + f0, acc);
-    if (lane == 0) degs[i] = deg * inv_kref;
 }
 
 // Backward edge phase: one warp per node i.  With dZ_ij = dS_i SiLU'(z_ij) / k_ref:
@@ -943,11 +975,12 @@ int forward(Surrogate &S, const SimView &v, bool training)
             e.fold_out = S.PQf;
             if ((rc = mm(S, st, S.A1[r], 2 * H, S.Wpq[r], H, n, 2 * H, H, e))) return rc;
         }
+        const int eb = std::min(nb(n, EWF / 16), S.sms * EDGE_BLOCKS);
         if (v.dim == 2)
-            k_edge_fwd<2><<<nb(n * 32, EWF), EWF, 0, st>>>(v.d, v.g, R2, inv2h, S.PQf, T + L.w3[r], invk, S.S[r],
+            k_edge_fwd<2><<<eb, EWF, 0, st>>>(v.d, v.g, R2, inv2h, S.PQf, T + L.w3[r], invk, S.S[r],
                                                            S.degs);
         else
-            k_edge_fwd<3><<<nb(n * 32, EWF), EWF, 0, st>>>(v.d, v.g, R2, inv2h, S.PQf, T + L.w3[r], invk, S.S[r],
+            k_edge_fwd<3><<<eb, EWF, 0, st>>>(v.d, v.g, R2, inv2h, S.PQf, T + L.w3[r], invk, S.S[r],
                                                            S.degs);
         CUR(cudaGetLastError());
         {
@@ -1196,6 +1229,13 @@ int sph_surrogate_init(sph_handle h, const double *weights, int64_t nweights, co
         S->n = v.n;
         S->npad = std::max(128, ((v.n + 127) / 128) * 128);
         S->L = L;
+        int dev = 0;
+        cudaError_t ce = cudaGetDevice(&dev);
+        if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&S->sms, cudaDevAttrMultiProcessorCount, dev);
+        if (ce != cudaSuccess) {
+            delete S;
+            return set_error(SPH_ECUDA, cudaGetErrorString(ce));
+        }
         int rc = alloc_surrogate(*S);
         if (rc) {
             delete S;
