@@ -23,6 +23,7 @@
 
 #include <cmath>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 using namespace sphgb;
@@ -33,7 +34,8 @@ namespace {
 constexpr int H = 128;        // hidden width
 constexpr int FIN = 16;       // padded node input width
 constexpr int FOUT = 16;      // padded output width
-constexpr int EW = 256;       // threads of the edge kernels (8 warps, one node each)
+constexpr int W3_SUMS = H * (2 * 3 + 3 + 1);   // edge weights and biases of a round, in 3-D
+constexpr int SUMS = 2 * W3_SUMS + 10 * H;     // and the biases of ten layers
 
 #define CUR(call)                                                                                  \
     do {                                                                                           \
@@ -110,6 +112,7 @@ struct Surrogate {
     // backward
     float *dYf, *dZf, *dA, *dh, *dS;
     bf16 *dYb, *dZb, *dAb, *dhb, *dPQ;
+    double *sums;                // FP64 sums over blocks: dW3 and db1 of both rounds, layer biases
     double *loss_d = nullptr;
     unsigned *err = nullptr;
     // judge snapshots (original order)
@@ -143,14 +146,6 @@ int dalloc(Surrogate &S, T **p, size_t count)
 
 // ---------------------------------------------------------------------------
 // Kernels
-
-// Derivative of SiLU with the fast reciprocal (relative error ~1e-6, far
-// below the BF16 rounding of the network's operands).
-__device__ __forceinline__ float dsilu(float z)
-{
-    const float s = __fdividef(1.f, 1.f + __expf(-z));
-    return s * (1.f + z * (1.f - s));
-}
 
 // The weights as the contractions read them, one launch for all tensors
 // (27 launches of 3 us each before): job y copies W (rows x cols of theta at
@@ -267,16 +262,6 @@ __device__ __forceinline__ bool edge_geom(const Dev &d, const Grid &g, float R2,
     return true;
 }
 
-__device__ __forceinline__ void load4(const __half *p, float (&v)[4])
-{
-    const uint2 raw = *(const uint2 *)p;
-    const float2 a = __half22float2(*(const __half2 *)&raw.x), b = __half22float2(*(const __half2 *)&raw.y);
-    v[0] = a.x;
-    v[1] = a.y;
-    v[2] = b.x;
-    v[3] = b.y;
-}
-
 __device__ __forceinline__ void store4(bf16 *p, const float (&v)[4])
 {
     __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
@@ -286,39 +271,6 @@ __device__ __forceinline__ void store4(bf16 *p, const float (&v)[4])
     *(uint2 *)p = raw;
 }
 
-
-// Width of a staged entry: 2 DIM + 3 edge features and the sender index,
-// padded to whole 16-byte vectors.
-template <int DIM>
-__host__ __device__ constexpr int slot_width() { return ((2 * DIM + 4) + 3) / 4 * 4; }
-
-// Lane-parallel decoding of up to 32 list entries of receiver i (entry
-// k0 + lane on each lane): the edge features and the sender of every valid
-// entry go to the warp's shared-memory slots; returns the ballot of valid
-// entries.
-template <int DIM>
-__device__ __forceinline__ unsigned stage_entries(const Dev &d, const Grid &g, float R2, float inv2h,
-                                                  const float4 &oi, int phi, const float4 &nfi, const float4 *NF,
-                                                  int i, int k0, int cnt, float (*slot)[slot_width<DIM>()])
-{
-    constexpr int NE = 2 * DIM + 3;
-    const int lane = threadIdx.x & 31;
-    const int k = k0 + lane;
-    bool valid = false;
-    if (k < cnt) {
-        int j;
-        float ef[NE];
-        valid = edge_features<DIM>(d, g, R2, inv2h, oi, phi, nfi, NF, d.nbr[(size_t)k * d.n + i], j, ef);
-        if (valid) {
-#pragma unroll
-            for (int c = 0; c < NE; ++c) slot[lane][c] = ef[c];
-            slot[lane][NE] = __int_as_float(j);
-        }
-    }
-    const unsigned mask = __ballot_sync(0xffffffffu, valid);
-    __syncwarp();
-    return mask;
-}
 
 __device__ __forceinline__ __half2 tanh_h2(__half2 x)
 {
@@ -487,122 +439,267 @@ __global__ void __launch_bounds__(EWF, EDGE_BLOCKS)
     }
 }
 
-// Backward edge phase: one warp per node i.  With dZ_ij = dS_i SiLU'(z_ij) / k_ref:
-// dP_i = sum_j dZ_ij, dQ_i = sum_j dZ_ji (the neighbour relation is
-// symmetric, so node i gathers its own sender terms), dW3 += dZ_ij e_ij and
-// db1 += dP_i, reduced per block and added with atomics.
+// Two FP32 values in one 64-bit register, and the packed arithmetic on them
+// (each half rounds like the scalar operation).
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// SiLU'(z) of a pair, which may be held negated, with the fast reciprocal
+// (relative error about 1e-6, far below the BF16 rounding of the network's
+// operands).  Scalar but for the last product: packed sums here made the training
+// step 5 % slower (the packed pipe is the busy one).
+template <bool NEGATED>
+__device__ __forceinline__ f32x2 dsilu2(f32x2 z)
+{
+    float a, b;
+    unpack2(z, a, b);
+    const float sa = __fdividef(1.f, 1.f + __expf(NEGATED ? a : -a)), sb = __fdividef(1.f, 1.f + __expf(NEGATED ? b : -b));
+    const float ua = fmaf(NEGATED ? -a : a, 1.f - sa, 1.f), ub = fmaf(NEGATED ? -b : b, 1.f - sb, 1.f);
+    return mul2(pack2(sa, sb), pack2(ua, ub));
+}
+
+// Two FP16 pairs (four features) as two FP32 pairs.
+__device__ __forceinline__ void half4(uint2 raw, f32x2 (&v)[2])
+{
+    const float2 a = __half22float2(*(const __half2 *)&raw.x), b = __half22float2(*(const __half2 *)&raw.y);
+    v[0] = pack2(a.x, a.y);
+    v[1] = pack2(b.x, b.y);
+}
+
+// Backward edge phase: one warp per node i, four features (two FP32 pairs) a
+// lane.  With dZ_ij = dS_i SiLU'(z_ij) / k_ref: dP_i = sum_j dZ_ij, dQ_i = sum_j
+// dZ_ji (the neighbour relation is symmetric, so node i gathers its own sender
+// terms), dW3 += dZ_ij e_ij and db1 += dP_i.
+//
+// Bound by the FP32 pipe and, with the few warps its registers allow, by latency:
+// per edge and feature two nine-term dot products, two SiLU' and a nine-term
+// outer product, in FP32.  The arithmetic is on packed pairs (half the
+// instructions; z_ji is summed negated, so that the channels that change sign
+// with the direction use the same pair features); two edges at a time share
+// each read of W3 from shared memory (four wavefronts a channel) and the next
+// two's rows are on their way meanwhile; the edge features lie in the slots as
+// pairs (e, e).  Blocks are persistent: the weight gradient stays in registers over
+// all nodes of a warp and is reduced over the block once (once per eight nodes
+// before: 160 atomics a node on 1 280 addresses); the blocks' sums meet in FP64
+// (w3_sum: dW3 then db1, zeroed before), which k_sums_out rounds into the gradient.
+// Measured (GB300): a training step on 193 496 particles 13.76 -> 12.51 ms (two
+// launches of 4.86 ms with scalar arithmetic and a block reduction per eight
+// nodes).  Not kept: three blocks of 128 (12 warps instead of 8, 168 registers:
+// the same), two features a lane (half the registers, two or three times the
+// warps, but the per-edge work shared by half as many features: 3 to 19 %
+// longer), the dot or the outer products scalar (2 to 8 % longer).
+constexpr int EWB = 256;     // threads (8 warps, one node each at a time)
+constexpr int EWB_BLOCKS = 1;
+
+// Slots of the backward edge phase: the 2 DIM + 3 features twice each, then
+// the sender, padded to whole 16-byte vectors.
 template <int DIM>
-__global__ void __launch_bounds__(EW, 2) k_edge_bwd(Dev d, Grid g, float R2, float inv2h, const float4 *NF,
-                                                 const __half *PQ, const float *W3, float inv_kref, const float *dS,
-                                                 bf16 *dPQ, float *gW3, float *gb1)
+__host__ __device__ constexpr int bwd_slot_width() { return (2 * (2 * DIM + 3) + 1 + 3) / 4 * 4; }
+
+// What an edge reads of its sender: P_j, Q_j and dS_j (four features).
+struct SenderRow {
+    uint2 p, q;
+    ulonglong2 s;
+};
+
+template <int DIM>
+__global__ void __launch_bounds__(EWB, EWB_BLOCKS)
+    k_edge_bwd(Dev d, Grid g, float R2, float inv2h, const float4 *NF, const __half *__restrict__ PQ, const float *W3,
+               float inv_kref, const float *__restrict__ dS, bf16 *dPQ, double *w3_sum)
 {
     constexpr int NE = 2 * DIM + 3;
-    constexpr int SWD = slot_width<DIM>();
-    __shared__ __align__(16) float slots[EW / 32][32][SWD];
-    __shared__ float red[EW / 32][H * (NE + 1)];
-    __shared__ float4 sw[NE][32];
-    for (int t = threadIdx.x; t < NE * 32; t += EW) {
+    constexpr int SWD = bwd_slot_width<DIM>();
+    constexpr int WARPS = EWB / 32;
+    __shared__ __align__(16) float slots[WARPS][32][SWD];
+    __shared__ __align__(16) float4 sw[NE][32];
+    __shared__ float red[H * (NE + 1)];
+    for (int t = threadIdx.x; t < NE * 32; t += EWB) {
         const int c = t / 32, l = t % 32;
         sw[c][l] = make_float4(W3[(4 * l) * NE + c], W3[(4 * l + 1) * NE + c], W3[(4 * l + 2) * NE + c],
                                W3[(4 * l + 3) * NE + c]);
     }
+    for (int t = threadIdx.x; t < H * (NE + 1); t += EWB) red[t] = 0.f;
     __syncthreads();
-    const int wid = threadIdx.x >> 5;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int f0 = lane * 4;
-    float gw[4][NE];
-    float dP[4] = {0.f, 0.f, 0.f, 0.f}, dQ[4] = {0.f, 0.f, 0.f, 0.f};
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, f0 = lane * 4;
+    const int n = d.n;
+    float(*const slot)[SWD] = slots[wid];
+    const f32x2 ik2 = pack2(inv_kref, inv_kref), minus = pack2(-1.f, -1.f);
+    f32x2 gw[NE][2], gb[2] = {0ull, 0ull};
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int c = 0; c < NE; ++c) gw[c][0] = gw[c][1] = 0ull;
+    for (int i = blockIdx.x * WARPS + wid; i < n; i += gridDim.x * WARPS) {
+        f32x2 Pi[2], Qn[2], dSi[2], dP[2] = {0ull, 0ull}, dQ[2] = {0ull, 0ull};
+        half4(*(const uint2 *)(PQ + (size_t)i * 2 * H + f0), Pi);
+        half4(*(const uint2 *)(PQ + (size_t)i * 2 * H + H + f0), Qn);
 #pragma unroll
-        for (int c = 0; c < NE; ++c) gw[q][c] = 0.f;
-    if (i < d.n) {
-        float Pi[4], Qi[4], dSi[4];
-        load4(PQ + (size_t)i * 2 * H + f0, Pi);
-        load4(PQ + (size_t)i * 2 * H + H + f0, Qi);
-        const float4 ds4 = *(const float4 *)(dS + (size_t)i * H + f0);
-        dSi[0] = ds4.x * inv_kref;
-        dSi[1] = ds4.y * inv_kref;
-        dSi[2] = ds4.z * inv_kref;
-        dSi[3] = ds4.w * inv_kref;
+        for (int q = 0; q < 2; ++q) Qn[q] = mul2(Qn[q], minus);
+        {
+            const ulonglong2 t = *(const ulonglong2 *)(dS + (size_t)i * H + f0);
+            dSi[0] = mul2(t.x, ik2);
+            dSi[1] = mul2(t.y, ik2);
+        }
         const float4 oi = d.pos[i];
         const float4 nfi = NF[i];
         const int phi = rec_phase(oi.w);
         const int cnt = d.ncnt[i];
-        float(*slot)[SWD] = slots[wid];
-        for (int k0 = 0; k0 < cnt; k0 += 32) {
-            unsigned mask = stage_entries<DIM>(d, g, R2, inv2h, oi, phi, nfi, NF, i, k0, cnt, slot);
-            while (mask) {
-                constexpr int GB = 2;
-                int sl[GB];
-                float Pj[GB][4], Qj[GB][4];
-                float4 dSj[GB];
+        auto fetch = [&](int e) {
+            const size_t j = (size_t)__float_as_int(slot[e][2 * NE]);
+            SenderRow r;
+            r.p = *(const uint2 *)(PQ + j * 2 * H + f0);
+            r.q = *(const uint2 *)(PQ + j * 2 * H + H + f0);
+            r.s = *(const ulonglong2 *)(dS + j * H + f0);
+            return r;
+        };
+        // M edges of the batch from slot e on, their rows given
+        auto edges = [&](int e, const SenderRow *row, auto count) {
+            constexpr int M = decltype(count)::value;
+            f32x2 zi[M][2], zj[M][2];   // z_ij, -z_ji
 #pragma unroll
-                for (int t = 0; t < GB; ++t) {
-                    sl[t] = mask ? __ffs(mask) - 1 : -1;
-                    if (mask) mask &= mask - 1;
-                    if (sl[t] >= 0) {
-                        const size_t j = (size_t)__float_as_int(slot[sl[t]][NE]);
-                        load4(PQ + j * 2 * H + f0, Pj[t]);
-                        load4(PQ + j * 2 * H + H + f0, Qj[t]);
-                        dSj[t] = *(const float4 *)(dS + j * H + f0);
-                    }
-                }
+            for (int t = 0; t < M; ++t) {
+                f32x2 Pj[2], Qj[2];
+                half4(row[t].p, Pj);
+                half4(row[t].q, Qj);
 #pragma unroll
-                for (int t = 0; t < GB; ++t) {
-                    if (sl[t] < 0) break;
-                    float ef[NE];
-#pragma unroll
-                    for (int c = 0; c < NE; ++c) ef[c] = slot[sl[t]][c];
-                    const float dsj[4] = {dSj[t].x, dSj[t].y, dSj[t].z, dSj[t].w};
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float zij = Pi[q] + Qj[t][q], zji = Pj[t][q] + Qi[q];
-#pragma unroll
-                        for (int c = 0; c < NE; ++c) {
-                            // e_ji: the relative position and the state differences change
-                            // sign, the distance and the phase flag do not
-                            const float ec = ef[c];
-                            const float4 wc4 = sw[c][lane];
-                            const float wq = q == 0 ? wc4.x : q == 1 ? wc4.y : q == 2 ? wc4.z : wc4.w;
-                            zij = fmaf(wq, ec, zij);
-                            zji = fmaf(wq, (c < DIM || c >= DIM + 2) ? -ec : ec, zji);
-                        }
-                        const float dzij = dSi[q] * dsilu(zij);
-                        const float dzji = dsj[q] * inv_kref * dsilu(zji);
-                        dP[q] += dzij;
-                        dQ[q] += dzji;
-#pragma unroll
-                        for (int c = 0; c < NE; ++c) gw[q][c] = fmaf(dzij, ef[c], gw[q][c]);
-                    }
+                for (int q = 0; q < 2; ++q) {
+                    zi[t][q] = add2(Pi[q], Qj[q]);
+                    zj[t][q] = fma2(Pj[q], minus, Qn[q]);
                 }
             }
+#pragma unroll
+            for (int c = 0; c < NE; ++c) {
+                const ulonglong2 w = *(const ulonglong2 *)&sw[c][lane];
+#pragma unroll
+                for (int t = 0; t < M; ++t) {
+                    const f32x2 ec = *(const f32x2 *)&slot[e + t][2 * c];
+                    // e_ji: the relative position and the state differences change
+                    // sign, the distance and the phase flag do not
+                    const f32x2 en = c < DIM || c >= DIM + 2 ? ec : mul2(ec, minus);
+                    zi[t][0] = fma2(w.x, ec, zi[t][0]);
+                    zi[t][1] = fma2(w.y, ec, zi[t][1]);
+                    zj[t][0] = fma2(w.x, en, zj[t][0]);
+                    zj[t][1] = fma2(w.y, en, zj[t][1]);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < M; ++t) {
+                f32x2 di[2];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    di[q] = mul2(dSi[q], dsilu2<false>(zi[t][q]));
+                    dP[q] = add2(dP[q], di[q]);
+                    dQ[q] = fma2(mul2(q ? row[t].s.y : row[t].s.x, ik2), dsilu2<true>(zj[t][q]), dQ[q]);
+                }
+#pragma unroll
+                for (int c = 0; c < NE; ++c) {
+                    const f32x2 ec = *(const f32x2 *)&slot[e + t][2 * c];
+                    gw[c][0] = fma2(di[0], ec, gw[c][0]);
+                    gw[c][1] = fma2(di[1], ec, gw[c][1]);
+                }
+            }
+        };
+        for (int k0 = 0; k0 < cnt; k0 += 32) {
+            // decoding: the valid ones of 32 entries to the slots, in list order
             __syncwarp();
-        }
-        store4(dPQ + (size_t)i * 2 * H + f0, dP);
-        store4(dPQ + (size_t)i * 2 * H + H + f0, dQ);
-    }
-    // block reduction of dW3 and db1
+            int j = 0;
+            float ef[NE];
+            bool valid = false;
+            if (k0 + lane < cnt)
+                valid = edge_features<DIM>(d, g, R2, inv2h, oi, phi, nfi, NF, d.nbr[(size_t)(k0 + lane) * n + i], j, ef);
+            const unsigned m = __ballot_sync(0xffffffffu, valid);
+            if (valid) {
+                float *const s = slot[__popc(m & ((1u << lane) - 1u))];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-#pragma unroll
-        for (int c = 0; c < NE; ++c) red[wid][(f0 + q) * NE + c] = gw[q][c];
-        red[wid][H * NE + f0 + q] = dP[q];
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < H * (NE + 1); t += EW) {
-        float s = 0.f;
-        for (int w2 = 0; w2 < EW / 32; ++w2) s += red[w2][t];
-        if (s != 0.f) {
-            if (t < H * NE) atomicAdd(gW3 + t, s);
-            else atomicAdd(gb1 + (t - H * NE), s);
+                for (int c = 0; c < NE; ++c) *(f32x2 *)(s + 2 * c) = pack2(ef[c], ef[c]);
+                s[2 * NE] = __int_as_float(j);
+            }
+            __syncwarp();
+            const int have = __popc(m);
+            if (have == 0) continue;
+            SenderRow row[2] = {fetch(0), fetch(min(1, have - 1))};
+            int e = 0;
+            for (; e + 2 <= have; e += 2) {
+                const SenderRow next[2] = {fetch(min(e + 2, have - 1)), fetch(min(e + 3, have - 1))};
+                edges(e, row, std::integral_constant<int, 2>());
+                row[0] = next[0];
+                row[1] = next[1];
+            }
+            if (e < have) edges(e, row, std::integral_constant<int, 1>());
         }
+        float p[4], q[4];
+        unpack2(dP[0], p[0], p[1]);
+        unpack2(dP[1], p[2], p[3]);
+        unpack2(dQ[0], q[0], q[1]);
+        unpack2(dQ[1], q[2], q[3]);
+        store4(dPQ + (size_t)i * 2 * H + f0, p);
+        store4(dPQ + (size_t)i * 2 * H + H + f0, q);
+        gb[0] = add2(gb[0], dP[0]);
+        gb[1] = add2(gb[1], dP[1]);
+    }
+    // block sums of dW3 and db1, warp after warp
+    for (int w = 0; w < WARPS; ++w) {
+        if (wid == w) {
+            float v[4];
+#pragma unroll
+            for (int c = 0; c < NE; ++c) {
+                unpack2(gw[c][0], v[0], v[1]);
+                unpack2(gw[c][1], v[2], v[3]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) red[(f0 + q) * NE + c] += v[q];
+            }
+            unpack2(gb[0], v[0], v[1]);
+            unpack2(gb[1], v[2], v[3]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) red[H * NE + f0 + q] += v[q];
+        }
+        __syncthreads();
+    }
+    for (int t = threadIdx.x; t < H * (NE + 1); t += EWB) {
+        const float s = red[t];
+        if (s != 0.f) atomicAdd(w3_sum + t, (double)s);
     }
 }
 
-// Column sums over n rows of src (ld), optionally weighted per row, added to dst.
-__global__ void k_colsum(const float *src, int ld, int cols, int n, const float *roww, float *dst)
+// The FP64 sums (edge weights and biases, biases of the layers) into the gradient.
+struct SumTable {
+    int count, from[14], to[14], len[14];
+};
+__global__ void k_sums_out(const double *sum, float *grad, const __grid_constant__ SumTable t)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (k < t.len[j]) grad[t.to[j] + k] = (float)sum[t.from[j] + k];
+}
+
+// Column sums over n rows of src (ld), optionally weighted per row, added to
+// dst: a thread per column and block of rows; the blocks' FP32 sums meet in FP64,
+// so the result does not depend on the order they finish in.
+__global__ void k_colsum(const float *src, int ld, int cols, int n, const float *roww, double *dst)
 {
     const int c = threadIdx.x;
     const int rows_per = (n + gridDim.x - 1) / gridDim.x;
@@ -610,7 +707,7 @@ __global__ void k_colsum(const float *src, int ld, int cols, int n, const float 
     if (c >= cols) return;
     float s = 0.f;
     for (int r = r0; r < r1; ++r) s += (roww ? roww[r] : 1.f) * src[(size_t)r * ld + c];
-    if (s != 0.f) atomicAdd(dst + c, s);
+    if (s != 0.f) atomicAdd(dst + c, (double)s);
 }
 
 // Targets from the state after k plain steps (original order, instance
@@ -922,6 +1019,7 @@ int alloc_backward(Surrogate &S)
     e |= dalloc(S, &S.dhb, P * H);
     e |= dalloc(S, &S.dS, P * H);
     e |= dalloc(S, &S.dPQ, P * 2 * H);
+    e |= dalloc(S, &S.sums, SUMS);
     if (e) return SPH_ENOMEM;
     CUR(cudaDeviceSynchronize());
     return SPH_OK;
@@ -1044,9 +1142,27 @@ int backward(Surrogate &S, const SimView &v)
     const int cs_blocks = std::max(1, std::min(1024, nb(n, 512)));
     int rc = 0;
     CUR(cudaMemsetAsync(G, 0, sizeof(float) * L.total, st));
+    CUR(cudaMemsetAsync(S.sums, 0, sizeof(double) * SUMS, st));
+    // the FP64 sums: the edge phase's of both rounds, then H for each bias of a layer
+    SumTable out{};
+    int next = 2 * W3_SUMS;
+    auto sum_of = [&](int from, int to, int len) {
+        out.from[out.count] = from;
+        out.to[out.count] = to;
+        out.len[out.count++] = len;
+    };
+    auto bias_sum = [&](int to, int len) {
+        sum_of(next, to, len);
+        next += H;
+        return S.sums + next - H;
+    };
+    for (int r = 0; r < 2; ++r) {
+        sum_of(r * W3_SUMS, L.w3[r], H * L.ne);
+        sum_of(r * W3_SUMS + H * L.ne, L.b1[r], H);
+    }
     // decoder, layer 2
     if ((rc = wgrad(S, st, S.dYb, FOUT, FOUT, S.A2, H, H, G + L.dec2w, L.nout, H))) return rc;
-    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dYf, FOUT, L.nout, n, nullptr, G + L.dec2b);
+    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dYf, FOUT, L.nout, n, nullptr, bias_sum(L.dec2b, L.nout));
     {
         Epi e;
         e.act = 2;
@@ -1060,7 +1176,7 @@ int backward(Surrogate &S, const SimView &v)
     }
     // decoder, layer 1
     if ((rc = wgrad(S, st, S.dZb, H, H, S.hLb, H, H, G + L.dec1w, H, H))) return rc;
-    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, G + L.dec1b);
+    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, bias_sum(L.dec1b, H));
     {
         Epi e;
         e.Cf = S.dh;
@@ -1074,7 +1190,7 @@ int backward(Surrogate &S, const SimView &v)
         const bf16 *hb = r == 0 ? S.A1[0] : S.A1[1];   // h_r in BF16: left half of [h, M]
         // node MLP, layer 2 (residual: dh passes through)
         if ((rc = wgrad(S, st, S.dhb, H, H, S.G1[r], H, H, G + L.n2[r], H, H))) return rc;
-        k_colsum<<<cs_blocks, 256, 0, st>>>(S.dh, H, H, n, nullptr, G + L.n2b[r]);
+        k_colsum<<<cs_blocks, 256, 0, st>>>(S.dh, H, H, n, nullptr, bias_sum(L.n2b[r], H));
         {
             Epi e;
             e.act = 2;
@@ -1088,7 +1204,7 @@ int backward(Surrogate &S, const SimView &v)
         }
         // node MLP, layer 1 on [h, M]
         if ((rc = wgrad(S, st, S.dZb, H, H, S.A1[r], 2 * H, 2 * H, G + L.n1[r], H, 2 * H))) return rc;
-        k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, G + L.n1b[r]);
+        k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, bias_sum(L.n1b[r], H));
         {
             Epi e;
             e.Cf = S.dA;
@@ -1099,7 +1215,7 @@ int backward(Surrogate &S, const SimView &v)
         }
         // second edge layer, applied after the sum: M = S We2^T + degs be2
         if ((rc = wgrad(S, st, S.dAb + H, 2 * H, H, S.S[r], H, H, G + L.we2[r], H, H))) return rc;
-        k_colsum<<<cs_blocks, 256, 0, st>>>(S.dA + H, 2 * H, H, n, S.degs, G + L.be2[r]);
+        k_colsum<<<cs_blocks, 256, 0, st>>>(S.dA + H, 2 * H, H, n, S.degs, bias_sum(L.be2[r], H));
         {
             Epi e;
             e.Cf = S.dS;
@@ -1107,12 +1223,13 @@ int backward(Surrogate &S, const SimView &v)
             if ((rc = mm(S, st, S.dAb + H, 2 * H, S.We2T[r], H, n, H, H, e))) return rc;
         }
         // edge phase
+        const int wb = std::min(nb(n, EWB / 32), S.sms * EWB_BLOCKS);
         if (v.dim == 2)
-            k_edge_bwd<2><<<nb(n * 32, EW), EW, 0, st>>>(v.d, v.g, R2, inv2h, S.NF, S.PQ[r], T + L.w3[r], invk,
-                                                         S.dS, S.dPQ, G + L.w3[r], G + L.b1[r]);
+            k_edge_bwd<2><<<wb, EWB, 0, st>>>(v.d, v.g, R2, inv2h, S.NF, S.PQ[r], T + L.w3[r], invk,
+                                                         S.dS, S.dPQ, S.sums + r * W3_SUMS);
         else
-            k_edge_bwd<3><<<nb(n * 32, EW), EW, 0, st>>>(v.d, v.g, R2, inv2h, S.NF, S.PQ[r], T + L.w3[r], invk,
-                                                         S.dS, S.dPQ, G + L.w3[r], G + L.b1[r]);
+            k_edge_bwd<3><<<wb, EWB, 0, st>>>(v.d, v.g, R2, inv2h, S.NF, S.PQ[r], T + L.w3[r], invk,
+                                                         S.dS, S.dPQ, S.sums + r * W3_SUMS);
         CUR(cudaGetLastError());
         // first edge layer, node parts: P = h W1^T + b1, Q = h W2^T
         if ((rc = wgrad(S, st, S.dPQ, 2 * H, 2 * H, hb, 2 * H, H, G + L.w1[r], H, H, G + L.w2[r]))) return rc;
@@ -1132,7 +1249,7 @@ int backward(Surrogate &S, const SimView &v)
     }
     // encoder, layer 2
     if ((rc = wgrad(S, st, S.dhb, H, H, S.A0, H, H, G + L.enc2w, H, H))) return rc;
-    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dh, H, H, n, nullptr, G + L.enc2b);
+    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dh, H, H, n, nullptr, bias_sum(L.enc2b, H));
     {
         Epi e;
         e.act = 2;
@@ -1146,7 +1263,8 @@ int backward(Surrogate &S, const SimView &v)
     }
     // encoder, layer 1
     if ((rc = wgrad(S, st, S.dZb, H, H, S.X16, FIN, FIN, G + L.enc1w, H, L.nin))) return rc;
-    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, G + L.enc1b);
+    k_colsum<<<cs_blocks, 256, 0, st>>>(S.dZf, H, H, n, nullptr, bias_sum(L.enc1b, H));
+    k_sums_out<<<dim3(nb(W3_SUMS), out.count), 256, 0, st>>>(S.sums, G, out);
     CUR(cudaGetLastError());
     return SPH_OK;
 }
