@@ -52,6 +52,16 @@ struct PendingTiming {
     cudaEvent_t a, b;
 };
 
+// Particles an SM up to which the sweeps run in blocks of 64 threads and load
+// their neighbours' records a chunk ahead of use.  Small inputs are bound by
+// the latency of a particle's chain of gathers, and blocks of 256 leave SMs idle;
+// large ones by issue and the L1 data pipe, where fewer registers and more warps are
+// better.  A step with the small form against the other (us, GB300, 2-D / 3-D):
+// 9 k particles 32.7 / 96.5 (7 k) against 36.5 / 125.3, 45 k 38.5 against 42.8, 97 k
+// 113.7 against 121.4 (3-D), 140 k 137.8 against 139.4 (3-D), 150 k 58.9 against 54.9
+// (2-D), 193 k 173 against 160 (3-D): the line lies where the 2-D curves cross.
+constexpr int AHEAD_PER_SM = 640;
+
 // Block sizes the persistent kernel is compiled for.  Each size has two
 // register budgets: 64 registers a thread (up to 1024 resident threads an
 // SM) and 128 (up to 512 threads); a shape with at most 512 threads an SM
@@ -262,11 +272,14 @@ void sph_sim::enqueue_eval(int stage, const float *drho_in, double dt)
     Dev &d = buf[0];
     float4 *vel_s = stage == 2 ? d.velq : d.velp;
     const int stage1 = stage != 2;
+    const bool ahead = n <= AHEAD_PER_SM * sms;
     launch(KI_SWEEP_A, [&] {
         if (stage1) {
-            const int ta = SPH_SWEEP_A_THREADS;
-            if (dim == 2) k_sweep_a<2><<<blocks(n, ta), ta, 0, stream>>>(d, grid, phys, drho_in, stage1, vel_s);
-            else k_sweep_a<3><<<blocks(n, ta), ta, 0, stream>>>(d, grid, phys, drho_in, stage1, vel_s);
+            const int ta = ahead ? AHEAD_THREADS : SPH_SWEEP_A_THREADS;
+            using Fn = void (*)(Dev, Grid, Phys, const float *, int, float4 *);
+            static const Fn fn[2][2] = {{k_sweep_a<2, false>, k_sweep_a<2, true>},
+                                        {k_sweep_a<3, false>, k_sweep_a<3, true>}};
+            fn[dim - 2][ahead]<<<blocks(n, ta), ta, 0, stream>>>(d, grid, phys, drho_in, stage1, vel_s);
         } else {
             // warps for the mixed particles: up to eight blocks of eight per SM
             const int mb = std::max(1, std::min(blocks(n), 8 * std::max(sms, 1)));
@@ -275,16 +288,14 @@ void sph_sim::enqueue_eval(int stage, const float *drho_in, double dt)
         }
     });
     launch(KI_SWEEP_B, [&] {
-        const int tb = SPH_SWEEP_B_THREADS, nbb = blocks(n, tb);
-        if (dim == 2) {
-            if (stage == 0) k_sweep_b<2, 0><<<nbb, tb, 0, stream>>>(d, grid, phys, dt);
-            else if (stage == 1) k_sweep_b<2, 1><<<nbb, tb, 0, stream>>>(d, grid, phys, dt);
-            else k_sweep_b<2, 2><<<nbb, tb, 0, stream>>>(d, grid, phys, dt);
-        } else {
-            if (stage == 0) k_sweep_b<3, 0><<<nbb, tb, 0, stream>>>(d, grid, phys, dt);
-            else if (stage == 1) k_sweep_b<3, 1><<<nbb, tb, 0, stream>>>(d, grid, phys, dt);
-            else k_sweep_b<3, 2><<<nbb, tb, 0, stream>>>(d, grid, phys, dt);
-        }
+        const int tb = ahead ? AHEAD_THREADS : SPH_SWEEP_B_THREADS;
+        using Fn = void (*)(Dev, Grid, Phys, double);
+        static const Fn fn[2][3][2] = {
+            {{k_sweep_b<2, 0, false>, k_sweep_b<2, 0, true>}, {k_sweep_b<2, 1, false>, k_sweep_b<2, 1, true>},
+             {k_sweep_b<2, 2, false>, k_sweep_b<2, 2, true>}},
+            {{k_sweep_b<3, 0, false>, k_sweep_b<3, 0, true>}, {k_sweep_b<3, 1, false>, k_sweep_b<3, 1, true>},
+             {k_sweep_b<3, 2, false>, k_sweep_b<3, 2, true>}}};
+        fn[dim - 2][stage][ahead]<<<blocks(n, tb), tb, 0, stream>>>(d, grid, phys, dt);
     });
 }
 

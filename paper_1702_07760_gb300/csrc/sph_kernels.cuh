@@ -920,7 +920,10 @@ __device__ __forceinline__ void correct_particle(const Dev &d, const Grid &g, co
 // comes from its record (rec_vol) with the constants of its phase: own
 // (vol0, irho0) for the renormalisation, the other phase's (vol0_o,
 // irho0_o) for the colour gradient.
-template <int DIM, bool NC, bool MIXED>
+// AHEAD: the neighbours' records are loaded one chunk before their use, and
+// the list two (the sweeps of small inputs, AHEAD_PER_SM); otherwise only
+// the list is loaded ahead.
+template <int DIM, bool NC, bool MIXED, bool AHEAD>
 __device__ __forceinline__ void sweep_a_pairs(const Dev &d, const Grid &g, const Phys &ph, int i, const float4 &oi,
                                               int phi_, int renorm, float vol0, float irho0, float vol0_o,
                                               float irho0_o, float &s1, float &c1, float &s2, float &c2,
@@ -930,52 +933,91 @@ __device__ __forceinline__ void sweep_a_pairs(const Dev &d, const Grid &g, const
     const int n = d.n, cnt = d.ncnt[i];
     typename RO<NC, unsigned>::type col = d.nbr + i;
     typename RO<NC, float4>::type pos = d.pos;
+    float p1 = 0.f, p2 = 0.f;
+    auto term = [&](unsigned e, const float4 &oj) {
+        float rx, ry, rz;
+        const float r2 = entry_vec<DIM>(oi, oj, e, cs, rx, ry, rz);
+        // beyond the support (list entries in the skin) t clamps to 0 and
+        // every kernel term vanishes
+        const float r = pair_dist(r2);
+        const float t = kernel_t(inv_h, r);
+        const float t3 = t * t * t;
+        const float vdj = rec_vd(oj.w);
+        if (!MIXED || rec_phase(oj.w) == phi_) {
+            if (renorm) {
+                // W / alpha_d = t^4 (2q + 1)
+                const float w = t3 * t * fmaf(2.f * inv_h, r, 1.f);
+                p1 = fmaf(rec_vol(vdj, vol0, irho0), w, p1);
+                p2 = fmaf(vdj, w, p2);
+            }
+        } else {
+            const float vj = rec_vol(vdj, vol0_o, irho0_o);
+            const float cc = vj * vj * t3;
+            gx = fmaf(cc, rx, gx);
+            gy = fmaf(cc, ry, gy);
+            if (DIM == 3) gz = fmaf(cc, rz, gz);
+        }
+    };
     // the list holds whole chunks (padding entries feed zero terms)
     constexpr int CH = SPH_LIST_CHUNK;
     unsigned ec[CH];  // the first chunk lies inside the list storage (kmax >= CH) even when empty
 #pragma unroll
     for (int c = 0; c < CH; ++c) ec[c] = ld_list<NC>(col + (size_t)c * n);
-    for (int k0 = 0; k0 < cnt; k0 += CH) {
+    if constexpr (AHEAD) {
+        auto fetch = [&](unsigned &e) {
+            int j = (int)(e & NBR_IDX_MASK);
+            if (!SPH_IN_RANGE(d.flags, j, n)) e = pad_entry(j = i);
+            return ld<NC>(pos + j);
+        };
         unsigned en[CH];
-        const bool more = k0 + CH < cnt;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) en[c] = more ? ld_list<NC>(col + (size_t)(k0 + CH + c) * n) : 0u;
-        float p1 = 0.f, p2 = 0.f;
+        float4 oc[CH];
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
-            const unsigned e = ec[c];
-            const int j = (int)(e & NBR_IDX_MASK);
-            if (!SPH_IN_RANGE(d.flags, j, n)) continue;
-            const float4 oj = ld<NC>(pos + j);
-            float rx, ry, rz;
-            const float r2 = entry_vec<DIM>(oi, oj, e, cs, rx, ry, rz);
-            // beyond the support (list entries in the skin) t clamps to 0 and
-            // every kernel term vanishes
-            const float r = pair_dist(r2);
-            const float t = kernel_t(inv_h, r);
-            const float t3 = t * t * t;
-            const float vdj = rec_vd(oj.w);
-            if (!MIXED || rec_phase(oj.w) == phi_) {
-                if (renorm) {
-                    // W / alpha_d = t^4 (2q + 1)
-                    const float w = t3 * t * fmaf(2.f * inv_h, r, 1.f);
-                    p1 = fmaf(rec_vol(vdj, vol0, irho0), w, p1);
-                    p2 = fmaf(vdj, w, p2);
-                }
-            } else {
-                const float vj = rec_vol(vdj, vol0_o, irho0_o);
-                const float cc = vj * vj * t3;
-                gx = fmaf(cc, rx, gx);
-                gy = fmaf(cc, ry, gy);
-                if (DIM == 3) gz = fmaf(cc, rz, gz);
+            oc[c] = cnt > 0 ? fetch(ec[c]) : oi;
+            en[c] = CH < cnt ? ld_list<NC>(col + (size_t)(CH + c) * n) : 0u;
+        }
+        for (int k0 = 0; k0 < cnt; k0 += CH) {
+            float4 on[CH];
+            unsigned e2[CH];
+            const bool more = k0 + CH < cnt, more2 = k0 + 2 * CH < cnt;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) on[c] = more ? fetch(en[c]) : oi;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) e2[c] = more2 ? ld_list<NC>(col + (size_t)(k0 + 2 * CH + c) * n) : 0u;
+            p1 = p2 = 0.f;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) term(ec[c], oc[c]);
+            if (renorm) {
+                kahan_add(s1, c1, p1);
+                kahan_add(s2, c2, p2);
+            }
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                ec[c] = en[c];
+                oc[c] = on[c];
+                en[c] = e2[c];
             }
         }
-        if (renorm) {
-            kahan_add(s1, c1, p1);
-            kahan_add(s2, c2, p2);
-        }
+    } else {
+        for (int k0 = 0; k0 < cnt; k0 += CH) {
+            unsigned en[CH];
+            const bool more = k0 + CH < cnt;
 #pragma unroll
-        for (int c = 0; c < CH; ++c) ec[c] = en[c];
+            for (int c = 0; c < CH; ++c) en[c] = more ? ld_list<NC>(col + (size_t)(k0 + CH + c) * n) : 0u;
+            p1 = p2 = 0.f;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const int j = (int)(ec[c] & NBR_IDX_MASK);
+                if (!SPH_IN_RANGE(d.flags, j, n)) continue;
+                term(ec[c], ld<NC>(pos + j));
+            }
+            if (renorm) {
+                kahan_add(s1, c1, p1);
+                kahan_add(s2, c2, p2);
+            }
+#pragma unroll
+            for (int c = 0; c < CH; ++c) ec[c] = en[c];
+        }
     }
 }
 
@@ -986,7 +1028,7 @@ __device__ __forceinline__ void sweep_a_finish(const Dev &d, const Phys &ph, con
 
 // skip_mixed (stage 2): the particles with an other-phase neighbour are left
 // to the warp-per-particle pass (sweep_a_mixed_warp).
-template <int DIM, bool NC>
+template <int DIM, bool NC, bool AHEAD = false>
 __device__ __forceinline__ void sweep_a_one(const Dev &d, const Grid &g, const Phys &ph, const float *drho_in,
                                             int renorm, bool skip_mixed, float4 *vel_s, int i)
 {
@@ -1009,10 +1051,10 @@ __device__ __forceinline__ void sweep_a_one(const Dev &d, const Grid &g, const P
     // particles with no other-phase neighbour (the bulk) take the loop
     // without the per-pair phase test
     if (other)
-        sweep_a_pairs<DIM, NC, true>(d, g, ph, i, oi, phi_, renorm_i, vol0, irho0, vol0_o, irho0_o, s1, c1, s2, c2,
+        sweep_a_pairs<DIM, NC, true, AHEAD>(d, g, ph, i, oi, phi_, renorm_i, vol0, irho0, vol0_o, irho0_o, s1, c1, s2, c2,
                                      gx, gy, gz);
     else if (renorm_i)
-        sweep_a_pairs<DIM, NC, false>(d, g, ph, i, oi, phi_, 1, vol0, irho0, vol0_o, irho0_o, s1, c1, s2, c2, gx,
+        sweep_a_pairs<DIM, NC, false, AHEAD>(d, g, ph, i, oi, phi_, 1, vol0, irho0, vol0_o, irho0_o, s1, c1, s2, c2, gx,
                                       gy, gz);
     // at stage 2 a particle with no other-phase particle in its list keeps the
     // zero surface tensor that stage 1 wrote (no colour gradient either time)
@@ -1144,7 +1186,7 @@ __device__ __forceinline__ void prefetch_epilogue(const Dev &d, int k)
 // (Eq. ct_dist_2).  grad_i W_ij = cF t^3 r_ij with t = 1 - q/2; the common
 // factor cF is applied once per particle.
 // STAGE 0: rates only; 1: then the predictor; 2: then the corrector.
-template <int DIM, int STAGE, bool NC>
+template <int DIM, int STAGE, bool NC, bool AHEAD = false>
 __device__ __forceinline__ void sweep_b_one(const Dev &d, const Grid &g, const Phys &ph, double dt, int i)
 {
     const float4 oi = d.posv[i];
@@ -1172,69 +1214,109 @@ __device__ __forceinline__ void sweep_b_one(const Dev &d, const Grid &g, const P
     typename RO<NC, float4>::type posv = d.posv;
     typename RO<NC, float4>::type T4 = d.T4;
     typename RO<NC, float2>::type T2 = d.T2;
+    auto pair = [&](unsigned e, int j, const float4 &oj, const float4 &uj) {
+        float rx, ry, rz;
+        const float r2 = entry_vec<DIM>(oi, oj, e, cs, rx, ry, rz);
+        const bool oil_j = oj.w < 0.f;
+        const float vol_j = fabsf(oj.w);
+        // beyond the support (list entries in the skin) t clamps to 0 and
+        // every pair term below vanishes
+        const float r = pair_dist(r2);
+        const float t = kernel_t(inv_h, r);
+        const float t3 = t * t * t;
+        // m_j (P_i/rho_i^2 + P_j/rho_j^2) t^3 with the record's m_j P_j / rho_j^2
+        const float pt = ((oil_j ? mP_oil : mP_wat) + uj.w) * t3;
+        px = fmaf(pt, rx, px);
+        py = fmaf(pt, ry, py);
+        if (DIM == 3) pz = fmaf(pt, rz, pz);
+        const float ux = ui.x - uj.x, uy = ui.y - uj.y, uz = DIM == 3 ? ui.z - uj.z : 0.f;
+        const float vt = vol_j * t3;
+        const float s = (oil_j ? kv_oil : kv_wat) * vt * __fdividef(r2, r2 + ph.delta2);
+        vx = fmaf(s, ux, vx);
+        vy = fmaf(s, uy, vy);
+        if (DIM == 3) vz = fmaf(s, uz, vz);
+        float ur = __fmul_rn(ux, rx);
+        ur = fmaf(uy, ry, ur);
+        if (DIM == 3) ur = fmaf(uz, rz, ur);
+        dv = fmaf(vt, ur, dv);
+        if ((iface_i | (__float_as_uint(oj.w) & 1u)) != 0u) {
+            // interface pairs are few: the particle's own tensor is re-read
+            // here (an L1 hit) rather than held in six registers
+            const float4 Ti = ld<NC>(T4 + i);
+            const float2 Ti2 = DIM == 3 ? ld<NC>(T2 + i) : make_float2(0.f, 0.f);
+            const float4 Tj = ld<NC>(T4 + j);
+            if (DIM == 2) {
+                const float xx = Ti.x + Tj.x, xy = Ti.y + Tj.y, yy = Ti.z + Tj.z;
+                sx = fmaf(t3, fmaf(xy, ry, __fmul_rn(xx, rx)), sx);
+                sy = fmaf(t3, fmaf(yy, ry, __fmul_rn(xy, rx)), sy);
+            } else {
+                const float2 Tj2 = ld<NC>(T2 + j);
+                const float xx = Ti.x + Tj.x, xy = Ti.y + Tj.y, xz = Ti.z + Tj.z;
+                const float yy = Ti.w + Tj.w, yz = Ti2.x + Tj2.x, zz = Ti2.y + Tj2.y;
+                sx = fmaf(t3, fmaf(xz, rz, fmaf(xy, ry, __fmul_rn(xx, rx))), sx);
+                sy = fmaf(t3, fmaf(yz, rz, fmaf(yy, ry, __fmul_rn(xy, rx))), sy);
+                sz = fmaf(t3, fmaf(zz, rz, fmaf(yz, ry, __fmul_rn(xz, rx))), sz);
+            }
+        }
+    };
     // the list holds whole chunks (padding entries feed zero terms)
     constexpr int CH = SPH_LIST_CHUNK;
     unsigned ec[CH];  // the first chunk lies inside the list storage (kmax >= CH) even when empty
 #pragma unroll
     for (int c = 0; c < CH; ++c) ec[c] = ld_list<NC>(col + (size_t)c * n);
-    for (int k0 = 0; k0 < cnt; k0 += CH) {
+    if constexpr (AHEAD) {
+        // records one chunk ahead of their use, the list two (see sweep_a_pairs)
+        auto index = [&](unsigned &e) {
+            int j = (int)(e & NBR_IDX_MASK);
+            if (!SPH_IN_RANGE(d.flags, j, n)) e = pad_entry(j = i);
+            return j;
+        };
         unsigned en[CH];
-        const bool more = k0 + CH < cnt;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) en[c] = more ? ld_list<NC>(col + (size_t)(k0 + CH + c) * n) : 0u;
+        float4 oc[CH], uc[CH];
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
-            const unsigned e = ec[c];
-            const int j = (int)(e & NBR_IDX_MASK);
-            if (!SPH_IN_RANGE(d.flags, j, n)) continue;
-            const float4 oj = ld<NC>(posv + j);
-            const float4 uj = ld<NC>(vel_s + j);
-            float rx, ry, rz;
-            const float r2 = entry_vec<DIM>(oi, oj, e, cs, rx, ry, rz);
-            const bool oil_j = oj.w < 0.f;
-            const float vol_j = fabsf(oj.w);
-            // beyond the support (list entries in the skin) t clamps to 0 and
-            // every pair term below vanishes
-            const float r = pair_dist(r2);
-            const float t = kernel_t(inv_h, r);
-            const float t3 = t * t * t;
-            // m_j (P_i/rho_i^2 + P_j/rho_j^2) t^3 with the record's m_j P_j / rho_j^2
-            const float pt = ((oil_j ? mP_oil : mP_wat) + uj.w) * t3;
-            px = fmaf(pt, rx, px);
-            py = fmaf(pt, ry, py);
-            if (DIM == 3) pz = fmaf(pt, rz, pz);
-            const float ux = ui.x - uj.x, uy = ui.y - uj.y, uz = DIM == 3 ? ui.z - uj.z : 0.f;
-            const float vt = vol_j * t3;
-            const float s = (oil_j ? kv_oil : kv_wat) * vt * __fdividef(r2, r2 + ph.delta2);
-            vx = fmaf(s, ux, vx);
-            vy = fmaf(s, uy, vy);
-            if (DIM == 3) vz = fmaf(s, uz, vz);
-            float ur = __fmul_rn(ux, rx);
-            ur = fmaf(uy, ry, ur);
-            if (DIM == 3) ur = fmaf(uz, rz, ur);
-            dv = fmaf(vt, ur, dv);
-            if ((iface_i | (__float_as_uint(oj.w) & 1u)) != 0u) {
-                // interface pairs are few: the particle's own tensor is re-read
-                // here (an L1 hit) rather than held in six registers
-                const float4 Ti = ld<NC>(T4 + i);
-                const float2 Ti2 = DIM == 3 ? ld<NC>(T2 + i) : make_float2(0.f, 0.f);
-                const float4 Tj = ld<NC>(T4 + j);
-                if (DIM == 2) {
-                    const float xx = Ti.x + Tj.x, xy = Ti.y + Tj.y, yy = Ti.z + Tj.z;
-                    sx = fmaf(t3, fmaf(xy, ry, __fmul_rn(xx, rx)), sx);
-                    sy = fmaf(t3, fmaf(yy, ry, __fmul_rn(xy, rx)), sy);
-                } else {
-                    const float2 Tj2 = ld<NC>(T2 + j);
-                    const float xx = Ti.x + Tj.x, xy = Ti.y + Tj.y, xz = Ti.z + Tj.z;
-                    const float yy = Ti.w + Tj.w, yz = Ti2.x + Tj2.x, zz = Ti2.y + Tj2.y;
-                    sx = fmaf(t3, fmaf(xz, rz, fmaf(xy, ry, __fmul_rn(xx, rx))), sx);
-                    sy = fmaf(t3, fmaf(yz, rz, fmaf(yy, ry, __fmul_rn(xy, rx))), sy);
-                    sz = fmaf(t3, fmaf(zz, rz, fmaf(yz, ry, __fmul_rn(xz, rx))), sz);
-                }
+            const int j = cnt > 0 ? index(ec[c]) : i;
+            oc[c] = ld<NC>(posv + j);
+            uc[c] = ld<NC>(vel_s + j);
+            en[c] = CH < cnt ? ld_list<NC>(col + (size_t)(CH + c) * n) : 0u;
+        }
+        for (int k0 = 0; k0 < cnt; k0 += CH) {
+            float4 on[CH], un[CH];
+            unsigned e2[CH];
+            const bool more = k0 + CH < cnt, more2 = k0 + 2 * CH < cnt;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const int j = more ? index(en[c]) : i;
+                on[c] = ld<NC>(posv + j);
+                un[c] = ld<NC>(vel_s + j);
+            }
+#pragma unroll
+            for (int c = 0; c < CH; ++c) e2[c] = more2 ? ld_list<NC>(col + (size_t)(k0 + 2 * CH + c) * n) : 0u;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) pair(ec[c], (int)(ec[c] & NBR_IDX_MASK), oc[c], uc[c]);
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                ec[c] = en[c];
+                oc[c] = on[c];
+                uc[c] = un[c];
+                en[c] = e2[c];
             }
         }
+    } else {
+        for (int k0 = 0; k0 < cnt; k0 += CH) {
+            unsigned en[CH];
+            const bool more = k0 + CH < cnt;
 #pragma unroll
-        for (int c = 0; c < CH; ++c) ec[c] = en[c];
+            for (int c = 0; c < CH; ++c) en[c] = more ? ld_list<NC>(col + (size_t)(k0 + CH + c) * n) : 0u;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const int j = (int)(ec[c] & NBR_IDX_MASK);
+                if (!SPH_IN_RANGE(d.flags, j, n)) continue;
+                pair(ec[c], j, ld<NC>(posv + j), ld<NC>(vel_s + j));
+            }
+#pragma unroll
+            for (int c = 0; c < CH; ++c) ec[c] = en[c];
+        }
     }
     const float rho = by_phase(phi_, I.rho0) + d.drho_eval[i];
     float4 out;
@@ -1347,8 +1429,14 @@ static __global__ void __launch_bounds__(256, 4) k_build_list(Dev d, Grid g, Phy
 #ifndef SPH_SWEEP_A_THREADS
 #define SPH_SWEEP_A_THREADS 256
 #endif
-template <int DIM>
-static __global__ void __launch_bounds__(SPH_SWEEP_A_THREADS)
+// The sweeps of small inputs (AHEAD_PER_SM particles an SM): blocks of 64, so
+// that every SM gets a share, with up to 128 registers a thread for the
+// records they load ahead.
+constexpr int AHEAD_THREADS = 64, AHEAD_BLOCKS = 8;
+
+template <int DIM, bool AHEAD>
+static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_A_THREADS,
+                                         AHEAD ? AHEAD_BLOCKS : 1280 / SPH_SWEEP_A_THREADS)
     k_sweep_a(Dev d, Grid g, Phys ph, const float *__restrict__ drho_in, int stage1, float4 *vel_s)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1360,7 +1448,7 @@ static __global__ void __launch_bounds__(SPH_SWEEP_A_THREADS)
         d.clock[0] += d.clock[1];
         d.clock[1] = 0.0;
     }
-    sweep_a_one<DIM, true>(d, g, ph, drho_in, renorm, false, vel_s, i);
+    sweep_a_one<DIM, true, AHEAD>(d, g, ph, drho_in, renorm, false, vel_s, i);
 }
 
 // Warps [0, 8 mixed_blocks) of the launch take the mixed particles one at a
@@ -1394,21 +1482,19 @@ static __global__ void __launch_bounds__(256) k_sweep_a2(Dev d, Grid g, Phys ph,
     sweep_a_one<DIM, true>(d, g, ph, drho_in, 0, true, vel_s, i);
 }
 
-// Threads per block of the force sweep and the resident blocks per SM it is
-// compiled for (1024 threads an SM: up to 64 registers a thread).
+// Threads per block of the force sweep, compiled for 1024 threads an SM (up to
+// 64 registers a thread).
 #ifndef SPH_SWEEP_B_THREADS
 #define SPH_SWEEP_B_THREADS 256
 #endif
-#ifndef SPH_SWEEP_B_MIN_BLOCKS
-#define SPH_SWEEP_B_MIN_BLOCKS (1024 / SPH_SWEEP_B_THREADS)
-#endif
-template <int DIM, int STAGE>
-static __global__ void __launch_bounds__(SPH_SWEEP_B_THREADS, SPH_SWEEP_B_MIN_BLOCKS)
+template <int DIM, int STAGE, bool AHEAD>
+static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_B_THREADS,
+                                         AHEAD ? AHEAD_BLOCKS : 1024 / SPH_SWEEP_B_THREADS)
     k_sweep_b(Dev d, Grid g, Phys ph, double dt)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d.n) return;
-    sweep_b_one<DIM, STAGE, true>(d, g, ph, dt, i);
+    sweep_b_one<DIM, STAGE, true, AHEAD>(d, g, ph, dt, i);
 }
 
 // ---------------------------------------------------------------------------

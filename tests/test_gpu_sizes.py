@@ -1,0 +1,88 @@
+"""The forms a step takes by the size of its input: blocks of 64 threads that
+load their records ahead (up to 640 particles an SM, 97 280 on 152 SMs), blocks
+of 256 above; the one-kernel rebuild and graphs of several steps below that
+limit, the chain of kernels above it and under per-kernel timing; and the
+persistent kernel's two builds (up to 512 particles an SM, 77 824, and above).
+
+All of them do the same arithmetic per particle in the same order, so every
+form gives the same bits.
+"""
+import numpy as np
+import pytest
+
+from paper_1702_07760_gb300 import workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+FIELDS = ("pos", "vel", "rho", "order", "cell")
+
+
+@pytest.fixture(scope="module")
+def sphmod():
+    from paper_1702_07760_gb300 import build as B
+    from paper_1702_07760_gb300 import sph
+    B.build()
+    sph.load()
+    return sph
+
+
+def _same(a, b):
+    for f in FIELDS:
+        assert np.array_equal(a.read(f), b.read(f)), f
+    assert a.list_builds == b.list_builds and a.step_index == b.step_index
+
+
+# (2-D) one block, both sides of 77 824 (272 x 286 and 273 x 286 particles) and of 97 280
+# (311 x 312 and 312 x 312), with oil, walls and list rebuilds; (3-D) both sides of 97 280
+@pytest.mark.parametrize("shape", [(1, 2), (266, 280), (267, 280), (305, 306), (306, 306), (39, 40, 40), (40, 40, 40)])
+def test_every_form_gives_the_same_bits(sphmod, shape):
+    w = WL.drop_tank(len(shape), shape, drop_d_dx=min(shape) / 3, seed=sum(shape), perturb=True)
+    dt = WL.stable_dt(w.params)
+    graph, eager, timed, persistent = (sphmod.Simulation.from_workload(w) for _ in range(4))
+    graph.run(dt, 3)
+    graph.run(dt, 11)                  # a graph of eight steps and three of one
+    eager.run(dt, 14, graph=False)
+    timed.timing(True)
+    timed.run(dt, 14)
+    timed.timing(False)
+    persistent.run_persistent(dt, 14)
+    assert graph.list_builds >= 2 or min(shape) < 4
+    for s in (eager, timed, persistent):
+        _same(graph, s)
+    for s in (graph, eager, timed):    # a forced build and the sweeps of stage 0
+        s.timing(s is timed)
+        s.eval_rates()
+        s.timing(False)
+    for f in ("acc", "drho", "pressure", "rho_eval", "tensor"):
+        a = graph.read(f)
+        assert np.array_equal(a, eager.read(f)) and np.array_equal(a, timed.read(f)), f
+
+
+def test_periodic_and_piston_in_the_small_forms(sphmod):
+    w = WL.wave_tank_small()
+    m = w.meta["piston"]
+    dt = WL.stable_dt(w.params)
+    sims = [sphmod.Simulation.from_workload(w) for _ in range(3)]
+    for s in sims:
+        s.set_piston(m["axis"], m["amp"], m["omega"], m["phase"], m["t_end"])
+    sims[0].run(dt, 20)
+    sims[1].timing(True)
+    sims[1].run(dt, 20)
+    sims[2].run_persistent(dt, 20)
+    for s in sims[1:]:
+        _same(sims[0], s)
+        assert s.time == sims[0].time
+
+
+@pytest.mark.parametrize("block,grid", [(128, 4), (128, 9), (512, 3)])
+def test_chunks_beyond_the_warps(sphmod, block, grid):
+    """A grid with fewer warps than chunks of 32 particles: the first chunk of each warp is its
+    own, the others come from the counter."""
+    w = WL.drop_tank(2, (33, 41), drop_d_dx=10, seed=33, perturb=True)
+    dt = WL.stable_dt(w.params)
+    ref = sphmod.Simulation.from_workload(w)
+    ref.run(dt, 12)
+    s = sphmod.Simulation.from_workload(w)
+    s.set_launch_shape(block, grid, True)
+    s.run_persistent(dt, 12)
+    _same(ref, s)
