@@ -72,7 +72,7 @@ template <int DIM, int BS, int TPSM>
 __global__ void __launch_bounds__(BS, TPSM / BS) k_persistent_bs(Dev d, Dev scratch, Grid g, Phys ph, Sort s,
                                                                   GridBarrier *bar, double dt, int nsteps, int dyn)
 {
-    persistent_steps<DIM>(d, scratch, g, ph, s, bar, dt, nsteps, dyn);
+    persistent_steps<DIM, TPSM <= 512>(d, scratch, g, ph, s, bar, dt, nsteps, dyn);
 }
 
 using PersistFn = void (*)(Dev, Dev, Grid, Phys, Sort, GridBarrier *, double, int, int);
@@ -379,7 +379,7 @@ int sph_sim::persistent_shape(int bs, int grid_req, int *grid_out, PersistFn *fn
     int dev = 0, sms = 0, fit = 0;
     CU(cudaGetDevice(&dev));
     CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const bool wide = grid_req > 0 && bs * ((grid_req + sms - 1) / sms) <= 512;
+    const bool wide = grid_req > 0 ? bs * ((grid_req + sms - 1) / sms) <= 512 : (int64_t)n <= (int64_t)sms * 512;
     PersistFn fn = persist_fn(dim, bs, wide);
     CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, (const void *)fn, bs, 0));
     if (fit < 1) return fail(SPH_ECUDA, "the persistent kernel does not fit an SM");
