@@ -247,8 +247,8 @@ int sph_step(sph_handle h, double dt);
  * error.  With graph != 0 one step is captured once into a CUDA graph and
  * replayed: a one-thread kernel copies the device rebuild flag into the
  * condition of a conditional (IF) node whose body is the cell-list chain, so
- * steps without a list build launch five kernels instead of fourteen.  The
- * eager form (graph == 0) launches all fourteen, the cell-list kernels
+ * steps without a list build launch five kernels instead of thirteen.  The
+ * eager form (graph == 0) launches all thirteen, the cell-list kernels
  * returning at once without a build; both compute the same bits. */
 int sph_run(sph_handle h, double dt, int64_t nsteps, int graph);
 

@@ -38,13 +38,14 @@ int fail(int code, const std::string &msg)
     } while (0)
 
 enum KernelId {
-    KI_MEMSET, KI_HASH, KI_SCAN, KI_SCATTER, KI_RANK, KI_GATHER, KI_COPY, KI_LIST, KI_SWEEP_A, KI_SWEEP_B,
+    KI_MEMSET, KI_HASH, KI_SCAN, KI_SCATTER, KI_RANK, KI_GATHER, KI_LIST, KI_SWEEP_A, KI_SWEEP_B,
     KI_PERSISTENT, KI_COUNT
 };
+// neighbour_list includes the copy of the reordered state back from the scratch set;
 // sweep_b includes the predictor (stage 1) or the corrector (stage 2);
 // persistent_steps is one cooperative launch running whole steps
 const char *k_names[KI_COUNT] = {"count_reset", "cell_hash", "cell_scan", "cell_scatter",
-                                 "cell_rank", "reorder_gather", "reorder_copy", "neighbour_list",
+                                 "cell_rank", "reorder_gather", "neighbour_list",
                                  "sweep_a", "sweep_b", "persistent_steps"};
 
 struct PendingTiming {
@@ -271,13 +272,9 @@ void sph_sim::enqueue_build_cells(bool force)
         if (dim == 2) k_gather<2><<<blocks(n), 256, 0, stream>>>(s, t, grid, sort);
         else k_gather<3><<<blocks(n), 256, 0, stream>>>(s, t, grid, sort);
     });
-    launch(KI_COPY, [&] {
-        if (dim == 2) k_copy_back<2><<<blocks(n), 256, 0, stream>>>(t, s);
-        else k_copy_back<3><<<blocks(n), 256, 0, stream>>>(t, s);
-    });
     launch(KI_LIST, [&] {
-        if (dim == 2) k_build_list<2><<<blocks(n), 256, 0, stream>>>(s, grid, phys);
-        else k_build_list<3><<<blocks(n), 256, 0, stream>>>(s, grid, phys);
+        if (dim == 2) k_build_list<2><<<blocks(n), 256, 0, stream>>>(t, s, grid, phys);
+        else k_build_list<3><<<blocks(n), 256, 0, stream>>>(t, s, grid, phys);
     });
 }
 

@@ -727,9 +727,9 @@ __device__ __forceinline__ void copy_one(const Dev &src, const Dev &dst, int k)
 
 // Neighbour list of particle i: every j != i within 2h + 2 skin at the
 // positions of the build, so the list stays complete while no particle moves
-// farther than the skin.
+// farther than the skin.  tags: the particles' tags in sorted order.
 template <int DIM, bool NC>
-__device__ __forceinline__ void list_one(const Dev &d, const Grid &g, const Phys &ph, int i)
+__device__ __forceinline__ void list_one(const Dev &d, const Grid &g, const Phys &ph, const uint8_t *tags, int i)
 {
     const float4 oi = d.pos[i];
     const int phi_ = rec_phase(oi.w);
@@ -737,13 +737,13 @@ __device__ __forceinline__ void list_one(const Dev &d, const Grid &g, const Phys
     int other = 0;
     const int n = d.n, kmax = ph.kmax;
     unsigned *__restrict__ nbr = d.nbr;
-    typename RO<NC, uint8_t>::type tag = d.tag;
+    typename RO<NC, uint8_t>::type tag = tags;
     // a static boundary particle while every static boundary particle is at
     // rest: its pairs with the others feed the force sweep nothing (u_ij = 0,
     // and its own acceleration is not used), so they are written from the end
     // of its column backwards and then moved behind the rest of its list,
     // which the force sweep visits alone
-    const bool split = static_wall(d.tag[i]) && *(volatile unsigned *)d.walls_moving == 0u;
+    const bool split = static_wall(tags[i]) && *(volatile unsigned *)d.walls_moving == 0u;
     for_each_candidate<DIM, NC>(g, d.cstart, d.pos, d.cell[i], oi, ph.RL2, ph.RP,
         [&](int j, const float4 &oj, float, float, float, float, unsigned code) {
             if (j == i) return;
@@ -1408,21 +1408,18 @@ static __global__ void __launch_bounds__(256) k_gather(Dev src, Dev dst, Grid g,
     gather_one<DIM>(src, dst, g, s, k);
 }
 
+// Copies the reordered state back from the scratch set and builds the list: the
+// copy (90 bytes a particle, 17 us on 656 600 as a launch of its own) runs under
+// the list's instruction-bound scan, which needs nothing of the state but the tags,
+// read from the scratch set.
 template <int DIM>
-static __global__ void __launch_bounds__(256) k_copy_back(Dev src, Dev dst)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= src.n || !*dst.rebuild) return;
-    copy_one<DIM>(src, dst, k);
-}
-
-template <int DIM>
-static __global__ void __launch_bounds__(256, 4) k_build_list(Dev d, Grid g, Phys ph)
+static __global__ void __launch_bounds__(256, 4) k_build_list(Dev scratch, Dev d, Grid g, Phys ph)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d.n || !*d.rebuild) return;
     if (i == 0) *d.builds += 1;
-    list_one<DIM, true>(d, g, ph, i);
+    copy_one<DIM>(scratch, d, i);
+    list_one<DIM, true>(d, g, ph, scratch.tag, i);
 }
 
 // Threads per block of the stage-1 sweep A.
@@ -1686,10 +1683,11 @@ __device__ __forceinline__ void persistent_steps(Dev d, Dev scratch, Grid g, Phy
             if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
             for (int k = tid; k < n; k += stride) gather_one<DIM>(d, scratch, g, s, k);
             if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
-            for (int k = tid; k < n; k += stride) copy_one<DIM>(scratch, d, k);
-            if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
             if (tid == 0) *d.builds += 1;
-            for_each_particle(bar, n, dyn, [&](int i) { list_one<DIM, false>(d, g, ph, i); });
+            for_each_particle(bar, n, dyn, [&](int i) {
+                copy_one<DIM>(scratch, d, i);
+                list_one<DIM, false>(d, g, ph, scratch.tag, i);
+            });
             if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
         }
         // the step's first phase: everyone has the rebuild flag and the step counter (no phase
