@@ -244,12 +244,16 @@ int sph_eval_rates(sph_handle h);
 int sph_step(sph_handle h, double dt);
 
 /* nsteps steps of size dt, then waits for the stream and reports any device
- * error.  With graph != 0 one step is captured once into a CUDA graph and
- * replayed: a one-thread kernel copies the device rebuild flag into the
- * condition of a conditional (IF) node whose body is the cell-list chain, so
- * steps without a list build launch five kernels instead of thirteen.  The
- * eager form (graph == 0) launches all thirteen, the cell-list kernels
- * returning at once without a build; both compute the same bits. */
+ * error.  With graph != 0 the steps are replayed from a CUDA graph captured
+ * once per dt.  Up to 640 particles per SM a graph step is five kernels, the
+ * first a cooperative one that rebuilds the lists when the device rebuild flag
+ * is set and returns at once otherwise, and runs of eight steps and more
+ * replay eight to a graph.  Above that a one-thread kernel copies the flag
+ * into the condition of a conditional (IF) node whose body is the cell-list
+ * chain, so steps without a list build launch five kernels instead of
+ * thirteen.  The eager form (graph == 0) launches the same kernels, the
+ * cell-list ones returning at once without a build; all forms compute the
+ * same bits. */
 int sph_run(sph_handle h, double dt, int64_t nsteps, int graph);
 
 /* The same nsteps steps as sph_run in ONE cooperative kernel launch: every
@@ -268,10 +272,11 @@ int sph_run_persistent(sph_handle h, double dt, int64_t nsteps, int graph);
 /* Launch shape of sph_run_persistent: block in {128, 256, 512} threads,
  * grid_blocks blocks (clamped to what can be co-resident; 0 = as many as
  * can), and how each phase's particles are shared out: dynamic_chunks = 1
- * hands chunks of consecutive particles to warps from a grid-wide counter,
- * 0 gives each thread a fixed grid-stride share.  Shapes of at most 512
- * threads per SM run a build of the kernel with up to 128 registers a
- * thread, the others one with 64.  sph_get_launch_shape returns the shape
+ * hands chunks of consecutive particles to warps, the first by number and
+ * the rest from a grid-wide counter, 0 gives each thread a fixed grid-stride
+ * share.  Shapes of at most 512 threads per SM, and grid_blocks = 0 with at
+ * most 512 particles per SM, run a build of the kernel with up to 128
+ * registers a thread, the others one with 64.  sph_get_launch_shape returns the shape
  * with the grid it gives on the current device.  Default: 256, 0, 1. */
 int sph_set_launch_shape(sph_handle h, int block, int grid_blocks, int dynamic_chunks);
 int sph_get_launch_shape(sph_handle h, int *block, int *grid_blocks, int *dynamic_chunks);

@@ -63,6 +63,9 @@ struct PendingTiming {
 // (2-D), 193 k 173 against 160 (3-D): the line lies where the 2-D curves cross.
 constexpr int AHEAD_PER_SM = 640;
 
+// Steps in one graph of a small input.
+constexpr int STEPS_PER_GRAPH = 8;
+
 // Block sizes the persistent kernel is compiled for.  Each size has two
 // register budgets: 64 registers a thread (up to 1024 resident threads an
 // SM) and 128 (up to 512 threads); a shape with at most 512 threads an SM
@@ -143,7 +146,8 @@ struct sph_sim {
     int64_t t_launches[KI_COUNT] = {};
     double t_ms[KI_COUNT] = {};
     // per-launch graph of one step, replayed while dt matches
-    cudaGraphExec_t gexec = nullptr;
+    // (small inputs: also of several steps)
+    cudaGraphExec_t gexec = nullptr, gexec8 = nullptr;
     double gdt = 0.0;
     // persistent form: launch shape and its graph
     int pbs = 256, pgrid = 0;             // block size, grid blocks (0: as many as fit)
@@ -233,12 +237,15 @@ struct sph_sim {
     int blocks(int work, int threads = 256) const { return (work + threads - 1) / threads; }
     int sms = 0;  // multiprocessors of the device
 
+    // small inputs rebuild in one cooperative kernel of at most two blocks an SM (the per-kernel
+    // timing keeps the chain)
+    bool one_kernel_rebuild() const { return !timing && n <= AHEAD_PER_SM * sms; }
     void enqueue_build_cells(bool force);
     void enqueue_load(const double *x, const double *u, const double *rho, double check_dt);
     int enqueue_read(int kind, bool integer, void *out, size_t bytes, size_t staging_offset);
     void enqueue_eval(int stage, const float *drho_in, double dt);
     void enqueue_step(double dt);
-    int capture_step_graph(double dt);
+    int capture_step_graph(double dt, int steps, cudaGraphExec_t *out);
     int enqueue_set_state(const double *x, const double *u, const double *rho);
     int enqueue_run(double dt, int64_t nsteps, bool graph);
     int enqueue_read_state(double *x, double *u, double *rho);
@@ -256,6 +263,19 @@ void sph_sim::enqueue_build_cells(bool force)
     Dev &s = buf[0];
     Dev &t = buf[1];
     if (force) cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream);
+    if (one_kernel_rebuild()) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(std::min(blocks(n), 2 * sms));
+        cfg.blockDim = dim3(256);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        cudaLaunchKernelEx(&cfg, dim == 2 ? k_rebuild<2> : k_rebuild<3>, s, t, grid, phys, sort, bar);
+        return;
+    }
     launch(KI_MEMSET, [&] { k_zero<<<blocks(ncell), 256, 0, stream>>>(sort.count, ncell, rebuild); });
     launch(KI_HASH, [&] {
         if (dim == 2) k_hash<2><<<blocks(n), 256, 0, stream>>>(s, grid, sort);
@@ -324,13 +344,15 @@ namespace {
 __global__ void k_rebuild_cond(cudaGraphConditionalHandle h, const unsigned *rebuild);
 }  // namespace
 
-// The replayed step as a graph: a one-thread kernel reads the rebuild flag
-// into the condition of an IF node whose body is the cell-list chain, then
-// the four sweeps.  On steps without a rebuild the chain is not launched at
-// all (its kernels would return at once, but ten launches of n/256 blocks
-// still cost several microseconds each).  The body's kernels keep their own
-// flag test, so the graph and the eager sequence compute the same.
-int sph_sim::capture_step_graph(double dt)
+// The replayed step as a graph.  Small inputs (one_kernel_rebuild): `steps`
+// steps of five kernels, the first the rebuild in one kernel.  Otherwise one
+// step: a one-thread kernel reads the rebuild flag into the condition of an IF
+// node whose body is the cell-list chain, then the four sweeps.  On steps
+// without a rebuild the chain is not launched at all (its kernels would return
+// at once, but nine launches of n/256 blocks still cost several microseconds
+// each).  The body's kernels keep their own flag test, so the graph and the
+// eager sequence compute the same.
+int sph_sim::capture_step_graph(double dt, int steps, cudaGraphExec_t *out)
 {
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -350,6 +372,19 @@ int sph_sim::capture_step_graph(double dt)
         cudaGraphDestroy(g);
         return fail(SPH_ECUDA, std::string(what) + ": " + cudaGetErrorString(err));
     };
+    if (one_kernel_rebuild()) {
+        // no conditional node: the rebuild kernel returns at once on steps without a build
+        if ((e = cudaStreamBeginCaptureToGraph(stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
+            cudaSuccess)
+            return bail("graph capture", e);
+        for (int k = 0; k < steps; ++k) enqueue_step(dt);
+        if ((e = cudaStreamEndCapture(stream, &g)) != cudaSuccess) return bail("graph capture", e);
+        if ((e = cudaGraphInstantiate(&exec, g, 0)) != cudaSuccess) return bail("graph instantiate", e);
+        cudaGraphDestroy(g);
+        if (*out) cudaGraphExecDestroy(*out);
+        *out = exec;
+        return SPH_OK;
+    }
     if ((e = cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess)
         return bail("conditional handle", e);
     if ((e = cudaStreamBeginCaptureToGraph(stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
@@ -379,9 +414,8 @@ int sph_sim::capture_step_graph(double dt)
     if ((e = cudaStreamEndCapture(stream, &g)) != cudaSuccess) return bail("graph capture", e);
     if ((e = cudaGraphInstantiate(&exec, g, 0)) != cudaSuccess) return bail("graph instantiate", e);
     cudaGraphDestroy(g);
-    if (gexec) cudaGraphExecDestroy(gexec);
-    gexec = exec;
-    gdt = dt;
+    if (*out) cudaGraphExecDestroy(*out);
+    *out = exec;
     return SPH_OK;
 }
 
@@ -1554,11 +1588,28 @@ int sph_sim::enqueue_run(double dt, int64_t nsteps, bool graph)
     if (dt != last_dt) CU(cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream));
     last_dt = dt;
     if (use_graph) {
-        if (!gexec || gdt != dt) {
-            const int rc = capture_step_graph(dt);
+        if (gdt != dt) {
+            if (gexec) cudaGraphExecDestroy(gexec);
+            if (gexec8) cudaGraphExecDestroy(gexec8);
+            gexec = gexec8 = nullptr;
+            gdt = dt;
+        }
+        int64_t k = 0;
+        if (one_kernel_rebuild() && nsteps >= STEPS_PER_GRAPH) {
+            if (!gexec8) {
+                const int rc = capture_step_graph(dt, STEPS_PER_GRAPH, &gexec8);
+                if (rc != SPH_OK) return rc;
+            }
+            for (; k + STEPS_PER_GRAPH <= nsteps; k += STEPS_PER_GRAPH) {
+                CU(cudaGraphLaunch(gexec8, stream));
+                step += STEPS_PER_GRAPH;
+            }
+        }
+        if (k < nsteps && !gexec) {
+            const int rc = capture_step_graph(dt, 1, &gexec);
             if (rc != SPH_OK) return rc;
         }
-        for (int64_t k = 0; k < nsteps; ++k) {
+        for (; k < nsteps; ++k) {
             CU(cudaGraphLaunch(gexec, stream));
             step += 1;
         }
@@ -2034,6 +2085,7 @@ void sph_destroy(sph_handle s)
     s->collect_timing();
     for (auto e : s->free_events) cudaEventDestroy(e);
     if (s->gexec) cudaGraphExecDestroy(s->gexec);
+    if (s->gexec8) cudaGraphExecDestroy(s->gexec8);
     if (s->pexec) cudaGraphExecDestroy(s->pexec);
     for (void *p : s->allocs) cudaFree(p);
     if (s->own_stream) cudaStreamDestroy(s->stream);
