@@ -119,6 +119,8 @@ struct Surrogate {
     cudaEvent_t join[2] = {nullptr, nullptr};
     double *sums;                // FP64 sums over blocks: dW3 and db1 of both rounds, layer biases
     double *loss_d = nullptr;
+    double *loss_h = nullptr;    // pinned: where the loss and the gradient are read back
+    float *grad_h = nullptr;
     unsigned *err = nullptr;
     // judge snapshots (original order)
     double *sx = nullptr, *su = nullptr, *sr = nullptr;
@@ -134,6 +136,7 @@ struct Surrogate {
         for (cudaStream_t t : side)
             if (t) cudaStreamSynchronize(t);
         for (void *p : allocs) cudaFree(p);
+        if (loss_h) cudaFreeHost(loss_h);
         for (cudaEvent_t e : fork) cudaEventDestroy(e);
         for (cudaEvent_t e : join)
             if (e) cudaEventDestroy(e);
@@ -1051,6 +1054,13 @@ int alloc_backward(Surrogate &S)
             CUR(cudaEventCreateWithFlags(&S.join[k], cudaEventDisableTiming));
         }
     }
+    if (!S.loss_h) {
+        void *q = nullptr;
+        const cudaError_t ce = cudaMallocHost(&q, sizeof(double) + sizeof(float) * S.L.total);
+        if (ce != cudaSuccess) return set_error(SPH_ENOMEM, std::string("cudaMallocHost: ") + cudaGetErrorString(ce));
+        S.loss_h = static_cast<double *>(q);
+        S.grad_h = reinterpret_cast<float *>(S.loss_h + 1);
+    }
     e |= dalloc(S, &S.dS, P * H);
     if (e) return SPH_ENOMEM;
     CUR(cudaDeviceSynchronize());
@@ -1513,13 +1523,7 @@ int sph_surrogate_train_step(sph_handle h, const double *x1, const double *u1, c
     const SimView v = sim_view(h);
     if ((rc = forward(*S, v, true))) return rc;
     // count of (node, channel) terms: every channel of fluid nodes, the density channel of walls
-    // (computed on the device side by the loss kernel's mask; the host needs the wall count)
-    std::vector<uint8_t> tags(v.n);
-    CUR(cudaMemcpyAsync(tags.data(), v.d.tag, v.n, cudaMemcpyDeviceToHost, v.stream));
-    CUR(cudaStreamSynchronize(v.stream));
-    int64_t walls = 0;
-    for (uint8_t t : tags) walls += (t >> 1) & 1;
-    const double count = (double)(v.n - walls) * S->L.nout + (double)walls;
+    const double count = (double)(v.n - v.nwall) * S->L.nout + (double)v.nwall;
     CUR(cudaMemsetAsync(S->loss_d, 0, sizeof(double), v.stream));
     if (v.dim == 2)
         k_loss<2><<<nb(v.n), 256, 0, v.stream>>>(v.d, S->norm_d, S->t_jump, S->Y, x1, u1, rho1,
@@ -1540,16 +1544,13 @@ int sph_surrogate_train_step(sph_handle h, const double *x1, const double *u1, c
         CUR(cudaGetLastError());
         if ((rc = pack_weights(*S, v.stream))) return rc;
     }
-    double loss = 0.0;
-    CUR(cudaMemcpyAsync(&loss, S->loss_d, sizeof(double), cudaMemcpyDeviceToHost, v.stream));
-    if (grad_out) {
-        std::vector<float> g(ngrad);
-        CUR(cudaMemcpyAsync(g.data(), S->grad, sizeof(float) * ngrad, cudaMemcpyDeviceToHost, v.stream));
-        CUR(cudaStreamSynchronize(v.stream));
-        for (int64_t k = 0; k < ngrad; ++k) grad_out[k] = g[k];
-    }
+    // the loss and the gradient come back behind everything else, with one wait (check_err's)
+    CUR(cudaMemcpyAsync(S->loss_h, S->loss_d, sizeof(double), cudaMemcpyDeviceToHost, v.stream));
+    if (grad_out) CUR(cudaMemcpyAsync(S->grad_h, S->grad, sizeof(float) * ngrad, cudaMemcpyDeviceToHost, v.stream));
     if ((rc = check_err(*S, v.stream))) return rc;
-    if (loss_out) *loss_out = loss / count;
+    if (grad_out)
+        for (int64_t k = 0; k < ngrad; ++k) grad_out[k] = S->grad_h[k];
+    if (loss_out) *loss_out = *S->loss_h / count;
     return sim_check(h);
 }
 

@@ -121,6 +121,7 @@ struct sph_sim {
     double *clock = nullptr;              // device time, see Dev::clock
     Motion *motion = nullptr;             // device copy of the piston motion
     int64_t npiston = 0;                  // particles with wall == 2
+    int64_t nwall = 0;                    // particles with wall != 0
     bool moving = false;                  // a piston motion is set
     bool evaluated = false;               // acc holds a rates evaluation
     unsigned *amax = nullptr;             // per instance, max |a|^2 (FP32 bits) for sph_suggest_dt
@@ -1162,6 +1163,7 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
                 // bit 0 oil, bit 1 boundary (fixed or piston), bit 2 piston
                 tag[i] = (uint8_t)(phase[i] | (wall[i] ? 2 : 0) | (wall[i] == 2 ? 4 : 0));
                 s->npiston += wall[i] == 2;
+                s->nwall += wall[i] != 0;
                 iid[i] = (uint16_t)q;
             }
         if ((e = cudaMemcpyAsync(a0.tag, tag.data(), (size_t)n, cudaMemcpyHostToDevice, st)) != cudaSuccess)
@@ -1198,6 +1200,7 @@ SimView sim_view(sph_sim *s)
     v.h = s->P.h;
     v.rho0 = s->P.rho0;
     v.npiston = s->npiston;
+    v.nwall = s->nwall;
     return v;
 }
 

@@ -20,6 +20,7 @@ struct SimView {
     double h;
     const double *rho0;    // per-phase reference density of instance 0 (host)
     int64_t npiston;       // particles with a prescribed (piston) motion
+    int64_t nwall;         // boundary particles (fixed or piston)
 };
 
 int set_error(int code, const std::string &msg);
