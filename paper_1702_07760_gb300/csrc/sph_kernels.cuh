@@ -1438,10 +1438,14 @@ constexpr int AHEAD_THREADS = 64, AHEAD_BLOCKS = 8;
 // particles an SM, where it fills the ends of the sweeps (656 600 particles, 20
 // steps 8.51 -> 8.46 ms); small inputs were slower with it (9 380 particles 37.7 ->
 // 43.8 us a step).
-__device__ __forceinline__ void wait_for_launch_before()
+// Takes and returns the thread's index: what is read through it, read-only loads
+// included, cannot move above the wait.
+__device__ __forceinline__ int wait_for_launch_before(int i)
 {
     asm volatile("griddepcontrol.launch_dependents;");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("" : "+r"(i));
+    return i;
 }
 
 template <int DIM, bool AHEAD>
@@ -1449,8 +1453,7 @@ static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_A_THR
                                          AHEAD ? AHEAD_BLOCKS : 1280 / SPH_SWEEP_A_THREADS)
     k_sweep_a(Dev d, Grid g, Phys ph, const float *__restrict__ drho_in, int stage1, float4 *vel_s)
 {
-    wait_for_launch_before();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = wait_for_launch_before(blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= d.n) return;
     const int renorm = renorm_now(d, ph, stage1);
     // the lists built for this step are in place; the corrector decides the next build
@@ -1483,13 +1486,13 @@ template <int DIM>
 static __global__ void __launch_bounds__(256) k_sweep_a2(Dev d, Grid g, Phys ph, const float *__restrict__ drho_in,
                                                   float4 *vel_s, int mixed_blocks)
 {
-    wait_for_launch_before();
+    const int t = wait_for_launch_before(blockIdx.x * blockDim.x + threadIdx.x);
     if ((int)blockIdx.x < mixed_blocks) {
-        mixed_pass<DIM, true>(d, g, ph, drho_in, vel_s, (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                              (int)(mixed_blocks * blockDim.x) >> 5, (int)threadIdx.x & 31);
+        mixed_pass<DIM, true>(d, g, ph, drho_in, vel_s, t >> 5, (int)(mixed_blocks * blockDim.x) >> 5,
+                              (int)threadIdx.x & 31);
         return;
     }
-    const int i = (int)(blockIdx.x - mixed_blocks) * blockDim.x + threadIdx.x;
+    const int i = t - mixed_blocks * (int)blockDim.x;
     if (i >= d.n) return;
     sweep_a_one<DIM, true>(d, g, ph, drho_in, 0, true, vel_s, i);
 }
@@ -1504,8 +1507,7 @@ static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_B_THR
                                          AHEAD ? AHEAD_BLOCKS : 1024 / SPH_SWEEP_B_THREADS)
     k_sweep_b(Dev d, Grid g, Phys ph, double dt)
 {
-    wait_for_launch_before();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = wait_for_launch_before(blockIdx.x * blockDim.x + threadIdx.x);
     if (i >= d.n) return;
     sweep_b_one<DIM, STAGE, true, AHEAD>(d, g, ph, dt, i);
 }
