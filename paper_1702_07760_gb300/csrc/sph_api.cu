@@ -294,8 +294,8 @@ void sph_sim::enqueue_build_cells(bool force)
         else k_gather<3><<<blocks(n), 256, 0, stream>>>(s, t, grid, sort);
     });
     launch(KI_LIST, [&] {
-        if (dim == 2) k_build_list<2><<<blocks(n), 256, 0, stream>>>(t, s, grid, phys);
-        else k_build_list<3><<<blocks(n), 256, 0, stream>>>(t, s, grid, phys);
+        if (dim == 2) k_build_list<2><<<blocks(n, LIST_THREADS), LIST_THREADS, 0, stream>>>(t, s, grid, phys);
+        else k_build_list<3><<<blocks(n, LIST_THREADS), LIST_THREADS, 0, stream>>>(t, s, grid, phys);
     });
 }
 
