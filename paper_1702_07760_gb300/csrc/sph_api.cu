@@ -1201,8 +1201,11 @@ SimView sim_view(sph_sim *s)
     v.rho0 = s->P.rho0;
     v.npiston = s->npiston;
     v.nwall = s->nwall;
+    v.timing = s->timing;
     return v;
 }
+
+void sim_evaluated(sph_sim *s) { s->evaluated = true; }
 
 void sim_build_lists(sph_sim *s)
 {

@@ -21,12 +21,15 @@ struct SimView {
     const double *rho0;    // per-phase reference density of instance 0 (host)
     int64_t npiston;       // particles with a prescribed (piston) motion
     int64_t nwall;         // boundary particles (fixed or piston)
+    bool timing;           // per-kernel timing is on (nothing is replayed from a graph)
 };
 
 int set_error(int code, const std::string &msg);
 SimView sim_view(sph_sim *s);
 // Queues a cell and neighbour-list build at the current positions.
 void sim_build_lists(sph_sim *s);
+// Notes that a rates evaluation was queued by other means than sph_eval_rates.
+void sim_evaluated(sph_sim *s);
 // Waits for the stream and reports device error flags.
 int sim_check(sph_sim *s);
 // Adds `steps` to the host and device step counters and `elapsed` to the
