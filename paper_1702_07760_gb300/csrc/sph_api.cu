@@ -598,11 +598,27 @@ T *pinned_view(T *p)
 }
 
 // Queues the original-order copy of one field into `out`: in place when the
-// kernel can write it (device or managed memory), else through the staging
+// kernel can write it (device, managed or pinned memory), else through the staging
 // buffer (at staging_offset doubles) and a cudaMemcpyAsync.
 int sph_sim::enqueue_read(int kind, bool integer, void *out, size_t bytes, size_t staging_offset)
 {
     void *dst = device_view(out);
+    // pinned memory, its first and last element: vectors in whole lines where the start
+    // allows 16-byte stores, one double a particle as it is (contiguous across a
+    // warp).  What remains staged: tensors, integers, pageable or misaligned outputs.
+    const bool vec = kind == RK_X || kind == RK_U || kind == RK_ACC;
+    double *pin = dst || integer || kind == RK_T ? nullptr : pinned_view(static_cast<double *>(out));
+    if (pin && (uintptr_t)pin % (vec ? 16 : 8) == 0 &&
+        pinned_view(static_cast<double *>(out) + bytes / 8 - 1) == pin + bytes / 8 - 1) {
+        if (!vec) dst = pin;
+        else {
+            const int nb = blocks(n, RS_TILE);
+            if (dim == 2) k_read_lines<2><<<nb, RS_TILE, 0, stream>>>(D(), kind, pin);
+            else k_read_lines<3><<<nb, RS_TILE, 0, stream>>>(D(), kind, pin);
+            CU(cudaGetLastError());
+            return SPH_OK;
+        }
+    }
     double *fo = integer ? nullptr : (dst ? static_cast<double *>(dst) : read_buf + staging_offset);
     int *io = integer ? (dst ? static_cast<int *>(dst) : read_ibuf) : read_ibuf;
     if (dim == 2) k_unpermute<2><<<blocks(n), 256, 0, stream>>>(D(), kind, fo, io);
@@ -1849,10 +1865,11 @@ int sph_read(sph_handle s, int field, void *host_out, int64_t bytes)
 int sph_sim::enqueue_read_state(double *x, double *u, double *rho)
 {
     const size_t nn = (size_t)n, dd = (size_t)dim;
-    // pinned outputs (x and u on 16-byte boundaries): one kernel writes all
+    // pinned outputs (x and u on 16-byte boundaries, rho on 8): one kernel writes all
     // three in place, in whole lines
     double *px = pinned_view(x), *pu = pinned_view(u), *pr = pinned_view(rho);
-    if (px && pu && pr && ((uintptr_t)px % 16) == 0 && ((uintptr_t)pu % 16) == 0) {
+    if (px && pu && pr && ((uintptr_t)px % 16) == 0 && ((uintptr_t)pu % 16) == 0 &&
+        ((uintptr_t)pr % 8) == 0) {
         const int nb = blocks(n, RS_TILE);
         if (dim == 2) k_read_state_lines<2><<<nb, RS_TILE, 0, stream>>>(D(), px, pu, pr);
         else k_read_state_lines<3><<<nb, RS_TILE, 0, stream>>>(D(), px, pu, pr);
