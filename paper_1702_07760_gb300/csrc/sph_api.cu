@@ -1092,7 +1092,7 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
         err |= s->alloc(&s->sort.tile_sums, (size_t)s->ntiles);
         err |= s->alloc(&s->diag_out, (size_t)k * DIAG_STRIDE);
         err |= s->alloc(&s->diag_blk, diag_blk.size());
-        err |= s->alloc(&s->diag_part, diag_blk.size() * DIAG_SUMS);
+        err |= s->alloc(&s->diag_part, diag_blk.size() * DIAG_PART);
         err |= s->alloc(&s->diag_arrived, (size_t)k);
         err |= s->alloc(&s->diag_grav, 4);
         err |= s->alloc(&s->read_buf, N * 9 + 16);

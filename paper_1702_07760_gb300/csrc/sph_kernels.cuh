@@ -1979,78 +1979,130 @@ static __global__ void __launch_bounds__(RS_TILE) k_read_lines(Dev d, int kind, 
 // part[block] and the last block of an instance to finish (an arrival counter
 // per instance, reset by it) adds them up in block order.  Every sum is a
 // fixed tree, so the values do not depend on the order blocks finish in.
-// Bound by the FP64 pipe (1/64 of the FP32 rate; about 14 operations a fluid
-// particle) and the gathers through `inv`.  One block of 256 threads per
-// instance, which this replaces, left 151 of 152 SMs idle on a single
-// simulation: 6.94 ms on 656 600 particles (a call with the positions read
-// back 6.53 ms, now 0.26 ms, most of it the copy to the host).
+// Bound by the FP64 pipe (1/64 of the FP32 rate), so what need not be FP64 is
+// not: particles are counted in integers (the mass is the counts times the phases'
+// masses) and the largest |u|^2 is compared by its bits; a warp's eight
+// sums go down the butterfly halving their number at each step (9 additions a lane;
+// 55 for eleven sums one by one); blocks without a particle to add skip all of it.
+// 656 600 particles (GB300, profiler): sums 88 -> 51 us, covariance 32 -> 17 us; a call
+// with the positions read back 250 -> 193 us, 87 of them the copy to the host.
+// One block of 256 threads per instance left 151 of 152 SMs idle on a single
+// simulation: 6.94 ms on 656 600 particles.
 constexpr int DIAG_THREADS = 256;
 constexpr int DIAG_TILE = 4 * DIAG_THREADS;
 constexpr int DIAG_STRIDE = 20;
-constexpr int DIAG_SUMS = 11;   // mass, momentum, energies, oil sum, oil count; largest |u|^2
-constexpr int DIAG_COV = 6;
+constexpr int DIAG_SUMS = 8;   // momentum, energies, oil sum (the covariance: six, padded)
+constexpr int DIAG_PART = DIAG_SUMS + 3;   // words of a block's partials: the sums, water and oil counts, largest |u|^2
 
 struct DiagBlock {
     int inst;     // instance
     int index;    // this block's place among the instance's blocks
 };
 
-// Sums v[0 .. K-1] (the largest v[K-1] with MAX_LAST) over the block: a
-// butterfly in each warp, then the warps in order; the result in every lane
-// of warp 0.  sm: DIAG_THREADS / 32 * K doubles.
-template <int K, bool MAX_LAST>
-__device__ __forceinline__ void diag_reduce(double (&v)[K], double *sm)
+// What a thread, then a block, adds up.
+struct DiagSums {
+    double v[DIAG_SUMS];
+    long long water, oil;   // particles
+    long long umax2;        // bits of the largest |u|^2 (a finite or infinite value)
+};
+
+// Sums over the block; in thread 0 the result (INTS: of the integers too).
+// A warp's sums: at each of three steps a lane keeps one half of the columns and
+// sends the other, so lanes 4 c to 4 c + 3 end with column c; two steps more add
+// those four.  The warps' sums are added in order, a lane a column.
+template <bool INTS>
+__device__ __forceinline__ void diag_reduce(DiagSums &a)
 {
+    constexpr int WARPS = DIAG_THREADS / 32;
+    __shared__ double sm[WARPS][DIAG_SUMS];
+    __shared__ long long si[WARPS][3];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int c = 0; c < K; ++c) {
-        for (int o = 16; o > 0; o >>= 1) {
-            const double w = __shfl_xor_sync(0xffffffffu, v[c], o);
-            v[c] = MAX_LAST && c == K - 1 ? fmax(v[c], w) : v[c] + w;
+    for (int half = DIAG_SUMS / 2, o = 16; half > 0; half >>= 1, o >>= 1) {
+        const bool upper = lane & o;
+#pragma unroll
+        for (int c = 0; c < half; ++c) {
+            const double send = upper ? a.v[c] : a.v[c + half], keep = upper ? a.v[c + half] : a.v[c];
+            a.v[c] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
-        if (lane == 0) sm[wid * K + c] = v[c];
+    }
+    a.v[0] += __shfl_xor_sync(0xffffffffu, a.v[0], 2);
+    a.v[0] += __shfl_xor_sync(0xffffffffu, a.v[0], 1);
+    if ((lane & 3) == 0) sm[wid][lane >> 2] = a.v[0];
+    if (INTS) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a.water += __shfl_xor_sync(0xffffffffu, a.water, o);
+            a.oil += __shfl_xor_sync(0xffffffffu, a.oil, o);
+            a.umax2 = max(a.umax2, __shfl_xor_sync(0xffffffffu, a.umax2, o));
+        }
+        if (lane == 0) {
+            si[wid][0] = a.water;
+            si[wid][1] = a.oil;
+            si[wid][2] = a.umax2;
+        }
     }
     __syncthreads();
     if (wid == 0) {
+        if (lane < DIAG_SUMS) {
+            double t = sm[0][lane];
 #pragma unroll
-        for (int c = 0; c < K; ++c) {
-            double t = sm[c];
-            for (int w = 1; w < DIAG_THREADS / 32; ++w)
-                t = MAX_LAST && c == K - 1 ? fmax(t, sm[w * K + c]) : t + sm[w * K + c];
-            v[c] = t;
+            for (int w = 1; w < WARPS; ++w) t += sm[w][lane];
+            sm[0][lane] = t;
+        }
+        __syncwarp();
+        if (lane == 0) {
+#pragma unroll
+            for (int c = 0; c < DIAG_SUMS; ++c) a.v[c] = sm[0][c];
+            if (INTS)
+#pragma unroll
+                for (int w = 1; w < WARPS; ++w) {
+                    a.water += si[w][0];
+                    a.oil += si[w][1];
+                    a.umax2 = max(a.umax2, si[w][2]);
+                }
         }
     }
     __syncthreads();
 }
 
 // The block's partial values to part, and, in the last block of the instance
-// to arrive, the totals of all its blocks (true there).
-template <int K, bool MAX_LAST>
-__device__ __forceinline__ bool diag_total(double (&v)[K], double *sm, double *part, const DiagBlock &b, int nblocks,
+// to arrive, the totals of all its blocks (true there, in thread 0).  A block with
+// nothing to add (any: whether this thread added a particle) stores zeros.
+template <bool INTS>
+__device__ __forceinline__ bool diag_total(DiagSums &a, bool any, double *part, const DiagBlock &b, int nblocks,
                                            unsigned *arrived)
 {
     __shared__ bool s_last;
-    diag_reduce<K, MAX_LAST>(v, sm);
-    double *const mine = part + (size_t)blockIdx.x * K;
+    if (__syncthreads_or(any)) diag_reduce<INTS>(a);
     if (threadIdx.x == 0) {
+        double *const mine = part + (size_t)blockIdx.x * DIAG_PART;
 #pragma unroll
-        for (int c = 0; c < K; ++c) mine[c] = v[c];
+        for (int c = 0; c < DIAG_SUMS; ++c) mine[c] = a.v[c];
+        if (INTS) {
+            mine[DIAG_SUMS] = __longlong_as_double(a.water);
+            mine[DIAG_SUMS + 1] = __longlong_as_double(a.oil);
+            mine[DIAG_SUMS + 2] = __longlong_as_double(a.umax2);
+        }
         __threadfence();
         s_last = atomicAdd(arrived + b.inst, 1u) == (unsigned)nblocks - 1u;
     }
     __syncthreads();
     if (!s_last) return false;
     __threadfence();
-    const double *const all = part + (size_t)((int)blockIdx.x - b.index) * K;
+    const double *const all = part + (size_t)((int)blockIdx.x - b.index) * DIAG_PART;
+    a = DiagSums{};
+    for (int q = threadIdx.x; q < nblocks; q += DIAG_THREADS) {
+        const double *const p = all + (size_t)q * DIAG_PART;
 #pragma unroll
-    for (int c = 0; c < K; ++c) v[c] = 0.0;
-    for (int q = threadIdx.x; q < nblocks; q += DIAG_THREADS)
-#pragma unroll
-        for (int c = 0; c < K; ++c) {
-            const double w = __ldcg(all + (size_t)q * K + c);
-            v[c] = MAX_LAST && c == K - 1 ? fmax(v[c], w) : v[c] + w;
+        for (int c = 0; c < DIAG_SUMS; ++c) a.v[c] += __ldcg(p + c);
+        if (INTS) {
+            a.water += __double_as_longlong(__ldcg(p + DIAG_SUMS));
+            a.oil += __double_as_longlong(__ldcg(p + DIAG_SUMS + 1));
+            a.umax2 = max(a.umax2, __double_as_longlong(__ldcg(p + DIAG_SUMS + 2)));
         }
-    diag_reduce<K, MAX_LAST>(v, sm);
+    }
+    diag_reduce<INTS>(a);
     if (threadIdx.x == 0) arrived[b.inst] = 0u;
     return true;
 }
@@ -2060,14 +2112,11 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_sums(Dev d, const 
                                                             const double *grav, double *part, unsigned *arrived,
                                                             double *out)
 {
-    __shared__ double sm[DIAG_THREADS / 32 * DIAG_SUMS];
     const DiagBlock b = blk[blockIdx.x];
     const long long p0 = first[b.inst], p1 = first[b.inst + 1];
     const int nblocks = (int)((p1 - p0 + DIAG_TILE - 1) / DIAG_TILE);
     const Inst &I = d.inst[b.inst];
-    double acc[DIAG_SUMS];
-#pragma unroll
-    for (int c = 0; c < DIAG_SUMS; ++c) acc[c] = 0.0;
+    DiagSums a{};
     const long long base = p0 + (long long)b.index * DIAG_TILE + threadIdx.x;
 #pragma unroll
     for (int t = 0; t < DIAG_TILE / DIAG_THREADS; ++t) {
@@ -2078,32 +2127,36 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_sums(Dev d, const 
         const int tg = d.tag[k];
         if (tg & 2) continue;
         const int oil = tg & 1;
-        const double m = oil ? I.mass64[1] : I.mass64[0];
+        const double m = oil ? I.mass64[1] : I.mass64[0], hm = oil ? 0.5 * I.mass64[1] : 0.5 * I.mass64[0];
         double u2 = 0.0, gx = 0.0;
 #pragma unroll
         for (int c = 0; c < DIM; ++c) {
             const double uc = d.u[(size_t)c * d.n + k];
             const double xc = wrap_coord(d.x[(size_t)c * d.n + k], d.plo[c], d.period[c]) - I.offset[c];
-            acc[1 + c] += m * uc;
+            a.v[c] += m * uc;
             u2 += uc * uc;
             gx += grav[c] * xc;
-            if (oil) acc[6 + c] += xc;
+            if (oil) a.v[5 + c] += xc;
         }
-        acc[0] += m;
-        acc[4] += 0.5 * m * u2;
-        acc[5] -= m * gx;
-        acc[9] += oil;
-        acc[10] = fmax(acc[10], u2);
+        a.v[3] += hm * u2;
+        a.v[4] -= m * gx;
+        a.oil += oil;
+        a.water += 1 - oil;
+        // |u|^2 >= 0, so its bits are ordered as it is; a NaN, beyond infinity's bits or negative, does not count
+        const long long bits = __double_as_longlong(u2);
+        if (bits <= 0x7ff0000000000000LL) a.umax2 = max(a.umax2, bits);
     }
-    if (!diag_total<DIAG_SUMS, true>(acc, sm, part, b, nblocks, arrived)) return;
+    if (!diag_total<true>(a, a.water + a.oil > 0, part, b, nblocks, arrived)) return;
     if (threadIdx.x == 0) {
         double *o = out + (size_t)b.inst * DIAG_STRIDE;
+        const double oil = (double)a.oil;
+        o[0] = (double)a.water * I.mass64[0] + oil * I.mass64[1];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) o[c] = acc[c];
+        for (int c = 0; c < 5; ++c) o[1 + c] = a.v[c];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) o[6 + c] = acc[9] > 0.0 && c < DIM ? acc[6 + c] / acc[9] : 0.0;
-        o[9] = acc[9];
-        o[10] = sqrt(acc[10]);
+        for (int c = 0; c < 3; ++c) o[6 + c] = a.oil > 0 && c < DIM ? a.v[5 + c] / oil : 0.0;
+        o[9] = oil;
+        o[10] = sqrt(__longlong_as_double(a.umax2));
     }
 }
 
@@ -2111,16 +2164,14 @@ template <int DIM>
 static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_cov(Dev d, const long long *first, const DiagBlock *blk,
                                                            double *part, unsigned *arrived, double *out)
 {
-    __shared__ double sm[DIAG_THREADS / 32 * DIAG_COV];
     const DiagBlock b = blk[blockIdx.x];
     const long long p0 = first[b.inst], p1 = first[b.inst + 1];
     const int nblocks = (int)((p1 - p0 + DIAG_TILE - 1) / DIAG_TILE);
     const Inst &I = d.inst[b.inst];
     double *o = out + (size_t)b.inst * DIAG_STRIDE;
     const double cen[3] = {o[6], o[7], o[8]};
-    double cv[DIAG_COV];
-#pragma unroll
-    for (int c = 0; c < DIAG_COV; ++c) cv[c] = 0.0;
+    DiagSums a{};
+    bool any = false;
     const long long base = p0 + (long long)b.index * DIAG_TILE + threadIdx.x;
 #pragma unroll
     for (int t = 0; t < DIAG_TILE / DIAG_THREADS; ++t) {
@@ -2130,21 +2181,22 @@ static __global__ void __launch_bounds__(DIAG_THREADS) k_diag_cov(Dev d, const l
         if (!SPH_IN_RANGE(d.flags, k, d.n)) continue;
         const int tg = d.tag[k];
         if ((tg & 2) || !(tg & 1)) continue;
+        any = true;
         double r[3] = {0, 0, 0};
 #pragma unroll
         for (int c = 0; c < DIM; ++c)
             r[c] = wrap_coord(d.x[(size_t)c * d.n + k], d.plo[c], d.period[c]) - I.offset[c] - cen[c];
-        cv[0] += r[0] * r[0];
-        cv[1] += r[0] * r[1];
-        cv[2] += r[0] * r[2];
-        cv[3] += r[1] * r[1];
-        cv[4] += r[1] * r[2];
-        cv[5] += r[2] * r[2];
+        a.v[0] += r[0] * r[0];
+        a.v[1] += r[0] * r[1];
+        a.v[2] += r[0] * r[2];
+        a.v[3] += r[1] * r[1];
+        a.v[4] += r[1] * r[2];
+        a.v[5] += r[2] * r[2];
     }
-    if (!diag_total<DIAG_COV, false>(cv, sm, part, b, nblocks, arrived)) return;
+    if (!diag_total<false>(a, any, part, b, nblocks, arrived)) return;
     if (threadIdx.x == 0)
 #pragma unroll
-        for (int c = 0; c < DIAG_COV; ++c) o[11 + c] = cv[c];
+        for (int c = 0; c < 6; ++c) o[11 + c] = a.v[c];
 }
 
 }  // namespace sphgb
