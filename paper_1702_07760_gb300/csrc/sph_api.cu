@@ -63,6 +63,13 @@ struct PendingTiming {
 // (2-D), 193 k 173 against 160 (3-D): the line lies where the 2-D curves cross.
 constexpr int AHEAD_PER_SM = 640;
 
+// Particles an SM above which a sweep is launched while the one before it ends.
+// The dependent launch costs a fixed few us a sweep and fills the end of the sweep before.
+// 20 steps with it against without (us, GB300): 116 k particles 2946 against 2642, 140 k 3147
+// against 2932 (3-D), 105 k 1175 against 1085 (2-D); 238 k 4075 against 4068, 375 k 5305 against
+// 5342, 657 k 8469 against 8514 (3-D).
+constexpr int OVERLAP_PER_SM = 1536;
+
 // Steps in one graph of a small input.
 constexpr int STEPS_PER_GRAPH = 8;
 
@@ -218,7 +225,7 @@ struct sph_sim {
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
-        cfg.numAttrs = overlap && !timing && n > AHEAD_PER_SM * sms ? 1 : 0;
+        cfg.numAttrs = overlap && !timing && n > OVERLAP_PER_SM * sms ? 1 : 0;
         cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
     }
 

@@ -1438,10 +1438,10 @@ constexpr int AHEAD_THREADS = 64, AHEAD_BLOCKS = 6;
 // Launches of the sweeps overlap: a sweep is started while the one before it
 // still runs (programmatic dependent launch) and waits here for its results.
 // Each sweep lets the next one start at once; the wait is for the whole grid before,
-// which itself has waited for the one before it.  Used above AHEAD_PER_SM
+// which itself has waited for the one before it.  Used above OVERLAP_PER_SM
 // particles an SM, where it fills the ends of the sweeps (656 600 particles, 20
-// steps 8.51 -> 8.46 ms); small inputs were slower with it (9 380 particles 37.7 ->
-// 43.8 us a step).
+// steps 8.51 -> 8.46 ms); smaller inputs were slower with it (9 380 particles 37.7 ->
+// 43.8 us a step, 116 424 132 -> 147).
 // Takes and returns the thread's index: what is read through it, read-only loads
 // included, cannot move above the wait.
 __device__ __forceinline__ int wait_for_launch_before(int i)

@@ -58,6 +58,22 @@ def test_every_form_gives_the_same_bits(sphmod, shape):
         assert np.array_equal(a, eager.read(f)) and np.array_equal(a, timed.read(f)), f
 
 
+# both sides of 1 536 particles an SM (233 472 on 152 SMs; 486 x 480 and 487 x 480 particles),
+# above which a graph's sweeps start while the sweep before them ends
+@pytest.mark.parametrize("shape", [(480, 474), (481, 474)])
+def test_overlapped_sweeps_give_the_same_bits(sphmod, shape):
+    w = WL.drop_tank(2, shape, drop_d_dx=100, seed=sum(shape), perturb=True)
+    dt = WL.stable_dt(w.params)
+    graph, eager, timed = (sphmod.Simulation.from_workload(w) for _ in range(3))
+    graph.run(dt, 14)
+    eager.run(dt, 14, graph=False)
+    timed.timing(True)
+    timed.run(dt, 14)
+    timed.timing(False)
+    for s in (eager, timed):
+        _same(graph, s)
+
+
 def test_periodic_and_piston_in_the_small_forms(sphmod):
     w = WL.wave_tank_small()
     m = w.meta["piston"]
