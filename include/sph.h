@@ -306,8 +306,9 @@ int sph_test_stall_barrier(sph_handle h);
 /* Copies a field (SPH_FIELD_*) into host memory in original particle order.
  * bytes must be at least the field's size (see the field list).  Device or
  * managed memory is written in place by the kernel that unpermutes the
- * field; host memory (pinned is fastest) through a staging copy.  Waits for
- * the stream. */
+ * field, and so is pinned host memory (positions, velocities and accelerations
+ * from a 16-byte boundary on, fields of one double a particle from an 8-byte one);
+ * other host memory goes through a staging copy.  Waits for the stream. */
 int sph_read(sph_handle h, int field, void *host_out, int64_t bytes);
 
 /* x, u (n*dim) and rho (n) in one call with one wait: the state as sph_read
