@@ -91,3 +91,55 @@ def test_gradient_sizes(env, shape):
         assert np.linalg.norm(g - gr) / np.linalg.norm(gr) < 2e-2
     # the same state again: only the order of the FP32 atomics differs
     assert np.linalg.norm(grads[1] - grads[0]) < 1e-5 * np.linalg.norm(gr)
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_weight_gradients_of_partly_filled_rows(env, dim):
+    """The decoder's gradient has 5 or 7 rows, so most lanes of the warps that store it have
+    none: each tensor with its own error, within the 3e-2 that BF16 operands leave an output."""
+    from test_gpu_surrogate import _case
+    torch, sph = env
+    w, norm, flat = _case(dim, 60 + dim)
+    rng = np.random.Generator(np.random.PCG64(61))
+    _, _, _, sd_out = SL.split_norm(norm, dim)[:4]
+    fl = (w.wall == 0)[:, None]
+    x1 = w.x + fl * rng.normal(0, 1, w.x.shape) * sd_out[:dim]
+    u1 = w.u + fl * rng.normal(0, 1, w.u.shape) * sd_out[dim:2 * dim]
+    r1 = w.rho + rng.normal(0, 1, w.n) * sd_out[2 * dim] * np.asarray(w.params["rho0"])[w.phase]
+    t = [torch.tensor(a, dtype=torch.float64, device="cuda") for a in (x1, u1, r1)]
+    sim = sph.Simulation.from_workload(w)
+    sim.surrogate_init(flat, norm)
+    _, g = sim.surrogate_train_step(*[a.data_ptr() for a in t], update=False, want_grad=True)
+    recv, send, E = O.graph(w.params, w.x, w.phase, w.u, w.rho, norm)
+    a, drdt = O.rates(w.params, w.x, w.u, w.rho, w.phase, w.wall)
+    X = O.node_features(w.params, w.u, w.rho, w.phase, w.wall, norm, a, drdt)
+    y, cache = O.forward(flat, dim, X, E, recv, send, 20.0 if dim == 2 else 80.0)
+    tt = O.targets(w.params, w.x, w.u, w.rho, x1, u1, r1, w.phase, norm, a, drdt)
+    _, dy = O.loss(y, tt, O.output_mask(dim, w.wall))
+    want = SL.unflatten(O.backward(flat, dim, cache, dy), dim)
+    got = SL.unflatten(g, dim)
+    for name in ("dec2.w", "enc1.w"):
+        assert np.linalg.norm(got[name] - want[name]) < 3e-2 * np.linalg.norm(want[name]), name
+
+
+@pytest.mark.parametrize("M", [5, 31, 33, 100])
+@pytest.mark.parametrize("N", [64, 128, 256])
+def test_ragged_rows_over_several_column_chunks(env, M, N):
+    """The general contraction with a last tile of few rows and several chunks of 16 columns a
+    warp; rows of an odd length and K = 48 keep it off the layer path."""
+    torch, sph = env
+    K = 48
+    g = torch.Generator().manual_seed(M * N)
+    A = (torch.randn(M, K, generator=g) * 0.5).to(torch.bfloat16)
+    B = (torch.randn(N, K, generator=g) * 0.5).to(torch.bfloat16)
+    dA, dB = A.cuda(), B.cuda()
+    C = torch.full((M + 1, N + 1), -7.0, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    sph.mm_bf16(dA.data_ptr(), K, dB.data_ptr(), K, C.data_ptr(), N + 1, M, N, K, 0, False,
+                torch.cuda.current_stream().cuda_stream, err.data_ptr())
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    assert torch.all(C[M] == -7.0) and torch.all(C[:, N] == -7.0)
+    ref = A.float() @ B.float().T
+    bound = (A.float().abs() @ B.float().abs().T) * (K * 2.0 ** -22) + 1e-30
+    assert torch.all((C[:M, :N].cpu() - ref).abs() <= bound)
