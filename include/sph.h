@@ -47,7 +47,8 @@ extern "C" {
 #define SPH_ECFL       -5  /* a particle moved farther in a step than the cell skin allows */
 #define SPH_EDOMAIN    -6  /* a particle left the box of the cell grid */
 #define SPH_ECAPACITY  -7  /* a particle has more neighbours than max_neighbours */
-#define SPH_ETIMEOUT   -8  /* a grid barrier of the persistent kernel gave up after one second */
+#define SPH_ETIMEOUT   -8  /* a grid barrier gave up after one second (any call that may build the
+                              lists or run the persistent kernel, or the call that waits for it) */
 #define SPH_EFALLBACK  -9  /* the judge rejected a surrogate jump; the state holds the plain
                               method's result (sph_surrogate_advance_judged), not a failure */
 #define SPH_EBOUNDS   -10  /* an index read from device data was out of range (reported by the
@@ -253,7 +254,14 @@ int sph_step(sph_handle h, double dt);
  * chain, so steps without a list build launch five kernels instead of
  * thirteen.  The eager form (graph == 0) launches the same kernels, the
  * cell-list ones returning at once without a build; all forms compute the
- * same bits. */
+ * same bits.
+ * The cooperative rebuild (up to 640 particles per SM: here, in sph_step,
+ * sph_build_cells, sph_eval_rates, the queries of neighbours and pairs and the
+ * surrogate's calls) waits at grid-wide barriers, each for one second at most.
+ * When one gives up, what is queued behind it returns at once without
+ * integrating or updating weights, the call that waits for the stream returns
+ * SPH_ETIMEOUT, and the barrier is reset; the state is that of the last whole
+ * step and the next call builds the lists anew. */
 int sph_run(sph_handle h, double dt, int64_t nsteps, int graph);
 
 /* The same nsteps steps as sph_run in ONE cooperative kernel launch: every
@@ -262,7 +270,8 @@ int sph_run(sph_handle h, double dt, int64_t nsteps, int graph);
  * barrier.  The results are bit-identical to sph_run's (same per-particle
  * arithmetic and summation order).  Every barrier wait gives up after one
  * second; the launch then returns early, the state is left partly advanced
- * and the call returns SPH_ETIMEOUT.  The launch uses the shape set by
+ * (its density may be that of a step begun), the call returns SPH_ETIMEOUT and
+ * the next one builds the lists anew.  The launch uses the shape set by
  * sph_set_launch_shape or chosen by sph_autotune (default: 256 threads, as
  * many blocks per SM as fit).  With graph != 0 the launch is captured into a
  * CUDA graph (re-captured when dt, nsteps or the shape changes).  Waits for
@@ -297,10 +306,11 @@ int sph_autotune(sph_handle h, double dt, int trial_steps, int *best_block, int 
 int sph_sync(sph_handle h);
 
 /* Test support for the barrier time-out (no counterpart in the paper): puts
- * the persistent kernel's grid barrier in a state that no arrival completes,
- * so that the next sph_run_persistent waits out its one-second limit in every
- * block and returns SPH_ETIMEOUT, after which the barrier is reset and runs
- * work again.  The state advanced by that call is undefined. */
+ * the handle's grid barrier in a state that no arrival completes, so that the
+ * next launch that uses it (sph_run_persistent, or up to 640 particles per SM
+ * a list build) waits out its one-second limit in every block and the call
+ * that waits for it returns SPH_ETIMEOUT, after which the barrier is reset and
+ * runs work again. */
 int sph_test_stall_barrier(sph_handle h);
 
 /* Copies a field (SPH_FIELD_*) into host memory in original particle order.

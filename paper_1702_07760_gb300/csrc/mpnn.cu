@@ -797,12 +797,12 @@ __global__ void k_loss(Dev d, const float *norm, float T, const float *Y, const 
 }
 
 // Applies the de-normalised increments: x += dx, u += du on fluid particles,
-// rho += drho on all.
+// rho += drho on all; nothing when the list build behind them gave up (stopped).
 template <int DIM>
 __global__ void k_apply(Dev d, const float *norm, float T, const float *Y)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= d.n) return;
+    if (k >= d.n || stopped(d)) return;
     constexpr int NIN = 2 * DIM + 4, NOUT = 2 * DIM + 1;
     const float *mu_out = norm + 2 * NIN, *sd_out = norm + 2 * NIN + NOUT;
     const uint8_t tg = d.tag[k];
@@ -854,12 +854,13 @@ __global__ void k_predict_out(Dev d, const float *norm, float T, const float *Y,
     out[(size_t)p * NOUT + 2 * DIM] = (double)(T * a.w + D[2 * DIM] * by_phase(tg & 1, I.rho0));
 }
 
-// Adam (Kingma & Ba 2015) with bias correction folded into the step size.
-__global__ void k_adam(float *theta, const float *g, float *m, float *v, int count, const StepArgs *args, float b1,
-                       float b2)
+// Adam (Kingma & Ba 2015) with bias correction folded into the step size; the weights
+// stay when the list build behind the gradient gave up (stopped).
+__global__ void k_adam(Dev d, float *theta, const float *g, float *m, float *v, int count, const StepArgs *args,
+                       float b1, float b2)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
+    if (k >= count || stopped(d)) return;
     const float lr_t = args->lr_t, eps_t = args->eps_t;
     const float gk = g[k];
     const float mk = b1 * m[k] + (1.f - b1) * gk;
@@ -1403,7 +1404,7 @@ int enqueue_train_step(sph_handle h, Surrogate &S, bool update)
     CUR(cudaGetLastError());
     if ((rc = backward(S, v))) return rc;
     if (!update) return SPH_OK;
-    k_adam<<<nb(S.L.total), 256, 0, v.stream>>>(S.theta, S.grad, S.m, S.v, S.L.total, S.args, (float)ADAM_B1,
+    k_adam<<<nb(S.L.total), 256, 0, v.stream>>>(v.d, S.theta, S.grad, S.m, S.v, S.L.total, S.args, (float)ADAM_B1,
                                                 (float)ADAM_B2);
     CUR(cudaGetLastError());
     return pack_weights(S, v.stream);
@@ -1620,7 +1621,9 @@ int sph_surrogate_train_step(sph_handle h, const double *x1, const double *u1, c
     if (grad_out)
         for (int64_t k = 0; k < ngrad; ++k) grad_out[k] = S->grad_h[k];
     if (loss_out) *loss_out = *S->loss_h / count;
-    return sim_check(h);
+    rc = sim_check(h);
+    if (update && rc == SPH_ETIMEOUT) S->adam_t = t - 1;   // no update was made
+    return rc;
 }
 
 int sph_snapshot(sph_handle h, double *x_dev, double *u_dev, double *rho_dev)

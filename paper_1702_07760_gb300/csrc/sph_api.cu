@@ -478,10 +478,17 @@ int sph_sim::check_flags()
     if (f == 0) return SPH_OK;
     CU(cudaMemsetAsync(flags, 0, sizeof(unsigned), stream));
     if (f & FLAG_TIMEOUT) {
-        // a block gave up at a barrier: start the next launch from a clean barrier
+        // a block gave up at a barrier: start the next launch from a clean barrier and new
+        // lists (without a last step size the next state given forces them too), and count
+        // the steps that the device has made
+        long long done = 0;
         CU(cudaMemsetAsync(bar, 0, sizeof(GridBarrier), stream));
+        CU(cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream));
+        CU(cudaMemcpyAsync(&done, dstep, sizeof(done), cudaMemcpyDeviceToHost, stream));
         CU(cudaStreamSynchronize(stream));
-        return fail(SPH_ETIMEOUT, "a grid barrier of the persistent kernel waited longer than one second");
+        last_dt = 0.0;
+        step = done;
+        return fail(SPH_ETIMEOUT, "a grid barrier (persistent kernel or one-kernel list rebuild) waited longer than one second");
     }
     // the most specific cause first: a step too large for the skin often
     // also sends particles out of the box or produces non-finite values
@@ -509,9 +516,9 @@ namespace {
 template <int DIM>
 __global__ void k_load_state(Dev d, Grid g, Phys ph, const double *x, const double *u, const double *rho,
                              double check_dt);
-__global__ void k_add_step(long long *step, long long k, double *clock, double elapsed)
+__global__ void k_add_step(Dev d, long long *step, long long k, double *clock, double elapsed)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
+    if (threadIdx.x == 0 && blockIdx.x == 0 && !stopped(d)) {
         *step += k;
         clock[1] += elapsed;
     }
@@ -1138,6 +1145,12 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
     if ((e = cudaMemsetAsync(s->dstep, 0, sizeof(long long), st)) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaMemsetAsync(s->dbuilds, 0, sizeof(long long), st)) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaMemsetAsync(a0.nmixed, 0, sizeof(int), st)) != cudaSuccess) return cuda_fail(e);
+    // empty lists in the first cell until the first build is through
+    if ((e = cudaMemsetAsync(a0.cell, 0, sizeof(int) * N, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = cudaMemsetAsync(a0.cstart, 0, sizeof(int) * ((size_t)ncell + 1), st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = cudaMemsetAsync(a0.ncnt, 0, sizeof(int) * N, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = cudaMemsetAsync(a0.nfcnt, 0, sizeof(int) * N, st)) != cudaSuccess) return cuda_fail(e);
+    if ((e = cudaMemsetAsync(a0.nflag, 0, N, st)) != cudaSuccess) return cuda_fail(e);
     {
         int dev = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return cuda_fail(e);
@@ -1240,7 +1253,7 @@ int sim_check(sph_sim *s) { return s->check_flags(); }
 int sim_moved(sph_sim *s, int64_t steps, double elapsed)
 {
     if (s->n > 0) {
-        k_add_step<<<1, 32, 0, s->stream>>>(s->dstep, (long long)steps, s->clock, elapsed);
+        k_add_step<<<1, 32, 0, s->stream>>>(s->D(), s->dstep, (long long)steps, s->clock, elapsed);
         CU(cudaGetLastError());
         CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
     }
@@ -1823,12 +1836,9 @@ int sph_autotune(sph_handle s, double dt, int trial_steps, int *best_block, int 
 int sph_test_stall_barrier(sph_handle s)
 {
     if (!s) return fail(SPH_EINVAL, "handle is NULL");
-    // with `count` at a value no arrival can reach from below, no block is the
-    // last to arrive: every block waits out its one-second limit and returns
-    int gsz = 0;
-    int rc = s->persistent_shape(s->pbs, s->pgrid, &gsz, nullptr);
-    if (rc) return rc;
-    const unsigned count = (unsigned)gsz;
+    // with `count` above every grid, no block is the last to arrive, whichever kernel uses
+    // the barrier: its blocks wait out the one-second limit and return
+    const unsigned count = 1u << 30;
     CU(cudaMemcpyAsync(&s->bar->count, &count, sizeof(count), cudaMemcpyHostToDevice, s->stream));
     CU(cudaStreamSynchronize(s->stream));
     return SPH_OK;
@@ -1940,7 +1950,10 @@ int64_t sph_neighbours(sph_handle s, int64_t *start, int32_t *list, int64_t cap)
     std::vector<int> hc(n), order(n);
     CU(cudaMemcpyAsync(hc.data(), cnt, sizeof(int) * n, cudaMemcpyDeviceToHost, s->stream));
     CU(cudaMemcpyAsync(order.data(), d.pid, sizeof(int) * n, cudaMemcpyDeviceToHost, s->stream));
+    unsigned f = 0;
+    CU(cudaMemcpyAsync(&f, s->flags, sizeof(f), cudaMemcpyDeviceToHost, s->stream));
     CU(cudaStreamSynchronize(s->stream));
+    if (f & FLAG_TIMEOUT) return s->check_flags();   // the cells are unfinished
     // rows in original id order
     std::vector<int64_t> sorted_start(n + 1, 0);
     for (int k = 0; k < n; ++k) sorted_start[k + 1] = sorted_start[k] + hc[k];

@@ -43,7 +43,7 @@ enum : unsigned {
     FLAG_NONFINITE = 2u,  // NaN/Inf in the state
     FLAG_SKIN = 4u,       // predictor displacement beyond the skin
     FLAG_LIST = 8u,       // a particle has more list neighbours than max_neighbours
-    FLAG_TIMEOUT = 16u,   // a grid barrier of the persistent kernel gave up waiting
+    FLAG_TIMEOUT = 16u,   // a grid barrier (persistent kernel, one-kernel rebuild) gave up waiting
     FLAG_BOUNDS = 32u,    // an index out of range (bounds-checked builds only)
 };
 constexpr unsigned FLAG_ERRORS = 63u;
@@ -725,6 +725,11 @@ __device__ __forceinline__ void copy_one(const Dev &src, const Dev &dst, int k)
     dst.iid[k] = src.iid[k];
 }
 
+// Whether a grid barrier of an earlier launch gave up: the lists may be unfinished, and
+// nothing is integrated until the host has reset the barrier.  (The lists that are there
+// hold valid indices at any time: empty ones from the creation on.)
+__device__ __forceinline__ bool stopped(const Dev &d) { return *d.flags & FLAG_TIMEOUT; }
+
 // Neighbour list of particle i: every j != i within 2h + 2 skin at the
 // positions of the build, so the list stays complete while no particle moves
 // farther than the skin.  tags: the particles' tags in sorted order.
@@ -1186,6 +1191,8 @@ __device__ __forceinline__ void prefetch_epilogue(const Dev &d, int k)
 // (Eq. ct_dist_2).  grad_i W_ij = cF t^3 r_ij with t = 1 - q/2; the common
 // factor cF is applied once per particle.
 // STAGE 0: rates only; 1: then the predictor; 2: then the corrector.
+// The launches of small inputs (AHEAD, not in the persistent kernel) follow the
+// one-kernel rebuild and do nothing when its barrier gave up.
 template <int DIM, int STAGE, bool NC, bool AHEAD = false>
 __device__ __forceinline__ void sweep_b_one(const Dev &d, const Grid &g, const Phys &ph, double dt, int i)
 {
@@ -1204,6 +1211,7 @@ __device__ __forceinline__ void sweep_b_one(const Dev &d, const Grid &g, const P
     // list) add exact zeros while those are at rest: u_ij = 0 in the
     // continuity term, and the acceleration of a boundary particle is not used
     const int n = d.n, cnt = ld<NC>(d.walls_moving) ? d.ncnt[i] : d.nfcnt[i];
+    if (NC && AHEAD && stopped(d)) return;
     if (STAGE != 0) prefetch_epilogue<DIM, STAGE>(d, i);
     // per-phase constants of the pair terms as registers (selected per pair):
     // m_j P_i / rho_i^2 for a water and an oil neighbour, and the viscous factors
@@ -1461,7 +1469,7 @@ static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_A_THR
     if (i >= d.n) return;
     const int renorm = renorm_now(d, ph, stage1);
     // the lists built for this step are in place; the corrector decides the next build
-    if (stage1 && i == 0) {
+    if (stage1 && i == 0 && !(AHEAD && stopped(d))) {
         *d.rebuild = 0u;
         d.clock[0] += d.clock[1];
         d.clock[1] = 0.0;
@@ -1554,61 +1562,73 @@ __device__ __forceinline__ unsigned atom_add_acq_rel_gpu(unsigned *p, unsigned v
     return old;
 }
 
-__device__ __forceinline__ void st_release_gpu(unsigned long long *p, unsigned long long v)
+__device__ __forceinline__ unsigned long long atom_cas_acq_rel_gpu(unsigned long long *p, unsigned long long expect,
+                                                                   unsigned long long v)
 {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+    unsigned long long old;
+    asm volatile("atom.acq_rel.gpu.global.cas.b64 %0, [%1], %2, %3;" : "=l"(old) : "l"(p), "l"(expect), "l"(v) : "memory");
+    return old;
 }
 
-// Generation of the barrier at the start of a launch (it cannot advance before
-// this block has arrived).
-__device__ __forceinline__ unsigned barrier_generation(const GridBarrier *b)
+// Start of a launch that uses the barrier: its state word goes to *state, in
+// shared memory (it cannot advance before this block has arrived, unless a block gave up).
+// False when a barrier has given up since the host last reset it: the launch must do nothing.
+__device__ __forceinline__ bool barrier_begin(const GridBarrier *b, unsigned long long *state)
 {
-    return (unsigned)(ld_acquire_gpu(&b->state) >> 32);
+    if (threadIdx.x == 0) *state = ld_acquire_gpu(&b->state);
+    __syncthreads();
+    return !((unsigned)*state & FLAG_TIMEOUT);
 }
 
 // Grid-wide barrier.  Thread 0 of each block arrives with a release-acquire
 // add (the block's writes, ordered before it by the block barrier, become
 // visible to whoever acquires later); the last block to arrive resets the
 // arrival and chunk counters and publishes the next generation together with
-// the error flags in one release store, which the others poll with acquire
-// loads.  Every thread keeps the generation in `gen`, so a barrier is two round
+// the error flags, which the others poll with acquire loads.  Every block keeps the
+// state word it saw last (*state, in shared memory), so a barrier is two round
 // trips to L2; with the generation read before the arrival, the flags after the
 // release and one more barrier a step, 45 736 particles took 59.8 us a step
 // instead of 38 (9 380 particles 60.8 instead of 35).
-// Returns the error flags as they stood when the last block arrived (the same
-// value in every block), plus FLAG_TIMEOUT if this block gave up waiting.
-__device__ __forceinline__ unsigned grid_sync(GridBarrier *b, unsigned *flags, unsigned &gen)
+//
+// A block that has waited a second publishes the next generation with
+// FLAG_TIMEOUT in its place.  Both publish by compare-and-swap on the state word, so
+// the first one decides and every block gets the same answer, the last to arrive
+// too: after a time-out no block enters the next phase, and the one that finished ends
+// complete.  Later launches find the flag in the state word (barrier_begin) and in
+// *flags until the host resets both.
+// Returns the error flags as they stood when the last block arrived, or the block gave
+// up (the same value in every block).
+__device__ __forceinline__ unsigned grid_sync(GridBarrier *b, unsigned *flags, unsigned long long *state)
 {
-    __shared__ unsigned s_snap;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const unsigned arrived = atom_add_acq_rel_gpu(&b->count, 1u);
-        unsigned snap;
-        if (arrived == gridDim.x - 1) {
-            snap = *(volatile unsigned *)flags;
+        const unsigned long long before = *state, next = ((before >> 32) + 1ull) << 32;
+        unsigned long long v;
+        if (atom_add_acq_rel_gpu(&b->count, 1u) == gridDim.x - 1) {
+            const unsigned long long open = next | *(volatile unsigned *)flags;
             atomicExch(&b->work, 0u);
             atomicExch(&b->count, 0u);
-            st_release_gpu(&b->state, ((unsigned long long)(gen + 1u) << 32) | snap);
-        } else {
-            unsigned long long v = ld_acquire_gpu(&b->state);
-            if ((unsigned)(v >> 32) == gen) {
-                const unsigned long long t0 = global_ns();
-                while ((unsigned)((v = ld_acquire_gpu(&b->state)) >> 32) == gen) {
-                    __nanosleep(20);
-                    if (global_ns() - t0 > 1000000000ull) {
+            v = atom_cas_acq_rel_gpu(&b->state, before, open);
+            if (v == before) v = open;
+        } else if ((v = ld_acquire_gpu(&b->state)) == before) {
+            const unsigned long long t0 = global_ns();
+            while ((v = ld_acquire_gpu(&b->state)) == before) {
+                __nanosleep(20);
+                if (global_ns() - t0 > 1000000000ull) {
+                    const unsigned long long late = next | *(volatile unsigned *)flags | FLAG_TIMEOUT;
+                    v = atom_cas_acq_rel_gpu(&b->state, before, late);
+                    if (v == before) {
+                        v = late;
                         atomicOr(flags, FLAG_TIMEOUT);
-                        v |= FLAG_TIMEOUT;
-                        break;
                     }
+                    break;
                 }
             }
-            snap = (unsigned)v;
         }
-        s_snap = snap;
+        *state = v;
     }
     __syncthreads();
-    gen += 1u;
-    return s_snap;
+    return (unsigned)*state;
 }
 
 // Calls f(i) for every particle i < n in chunks of consecutive particles (32 a
@@ -1660,7 +1680,7 @@ __device__ __forceinline__ void for_each_particle(GridBarrier *bar, int n, int d
 // returned.
 template <int DIM>
 __device__ __forceinline__ unsigned rebuild_phases(const Dev &d, const Dev &scratch, const Grid &g, const Phys &ph,
-                                                   const Sort &s, GridBarrier *bar, unsigned &gen, int dyn,
+                                                   const Sort &s, GridBarrier *bar, unsigned long long *state, int dyn,
                                                    unsigned stop)
 {
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1668,30 +1688,30 @@ __device__ __forceinline__ unsigned rebuild_phases(const Dev &d, const Dev &scra
     const int n = d.n;
     unsigned f;
     for (int c = tid; c < s.ncell; c += stride) s.count[c] = 0;
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     for (int k = tid; k < n; k += stride) hash_one<DIM>(d, g, s, k);
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     const int ntiles = (s.ncell + SCAN_TILE - 1) / SCAN_TILE;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
         const int tot = scan_tile(s.count, d.cstart, s.ncell, t);
         if (threadIdx.x == 0) s.tile_sums[t] = tot;
     }
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     if (blockIdx.x == 0) scan_tile_sums(s.tile_sums, ntiles, d.cstart, s.ncell);
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     for (int c = tid; c < s.ncell; c += stride) d.cstart[c] += s.tile_sums[c / SCAN_TILE];
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     for (int k = tid; k < n; k += stride) scatter_one(s, d.cstart, k);
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     for (int p = tid; p < n; p += stride) rank_one(s, d.pid, d.cstart, p);
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     for (int k = tid; k < n; k += stride) gather_one<DIM>(d, scratch, g, s, k);
-    if ((f = grid_sync(bar, d.flags, gen)) & stop) return f;
+    if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     if (tid == 0) *d.builds += 1;
-    for_each_particle(bar, n, dyn, [&](int i) {
-        copy_one<DIM>(scratch, d, i);
-        list_one<DIM, false>(d, g, ph, scratch.tag, i);
-    });
+    // the copy apart from the list, which reads nothing it writes: in one loop the 2-D build of
+    // 128 registers reloaded 272 spilled bytes (4 drops of a batch, 20 steps 820 us; apart 792)
+    for (int k = tid; k < n; k += stride) copy_one<DIM>(scratch, d, k);
+    for_each_particle(bar, n, dyn, [&](int i) { list_one<DIM, false>(d, g, ph, scratch.tag, i); });
     return f;
 }
 
@@ -1701,13 +1721,14 @@ __device__ __forceinline__ unsigned rebuild_phases(const Dev &d, const Dev &scra
 // 38.5 -> 28.1; 3-D, 64 736 99.8 -> 91.8).  A block reads the rebuild flag
 // once: nothing lowers it before the sweeps that follow.  Error flags of the
 // state do not stop it (as the chain of kernels runs through), only a barrier
-// that gave up.
+// that gave up, in this launch or in an earlier one; the sweeps that follow then
+// integrate nothing and leave the flag up (stopped).
 template <int DIM>
 static __global__ void __launch_bounds__(256, 2) k_rebuild(Dev d, Dev scratch, Grid g, Phys ph, Sort s, GridBarrier *bar)
 {
-    if (!*(volatile unsigned *)d.rebuild) return;
-    unsigned gen = barrier_generation(bar);
-    rebuild_phases<DIM>(d, scratch, g, ph, s, bar, gen, 0, FLAG_TIMEOUT);
+    __shared__ unsigned long long state;
+    if (!*(volatile unsigned *)d.rebuild || !barrier_begin(bar, &state)) return;
+    rebuild_phases<DIM>(d, scratch, g, ph, s, bar, &state, 0, FLAG_TIMEOUT);
 }
 
 // Body of the persistent kernel (instantiated per block size by the host
@@ -1720,13 +1741,15 @@ __device__ __forceinline__ void persistent_steps(Dev d, Dev scratch, Grid g, Phy
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int stride = gridDim.x * blockDim.x;
     const int n = d.n;
-    unsigned gen = barrier_generation(bar);
-    if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
+    __shared__ unsigned long long word;
+    unsigned long long *const state = &word;
+    if (!barrier_begin(bar, state)) return;
+    if (grid_sync(bar, d.flags, state) & FLAG_ERRORS) return;
     for (int step = 0; step < nsteps; ++step) {
         // every block reads the flag after the barrier that closed the last step
         if (*(volatile unsigned *)d.rebuild) {
-            if (rebuild_phases<DIM>(d, scratch, g, ph, s, bar, gen, dyn, FLAG_ERRORS) & FLAG_ERRORS) return;
-            if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
+            if (rebuild_phases<DIM>(d, scratch, g, ph, s, bar, state, dyn, FLAG_ERRORS) & FLAG_ERRORS) return;
+            if (grid_sync(bar, d.flags, state) & FLAG_ERRORS) return;
         }
         // the step's first phase: everyone has the rebuild flag and the step counter (no phase
         // before the corrector writes them), so only the clock is set here, for the pistons of the
@@ -1737,15 +1760,15 @@ __device__ __forceinline__ void persistent_steps(Dev d, Dev scratch, Grid g, Phy
             d.clock[1] = 0.0;
         }
         for_each_particle(bar, n, dyn, [&](int i) { sweep_a_one<DIM, false, AHEAD>(d, g, ph, d.drho, renorm, false, d.velp, i); });
-        if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
+        if (grid_sync(bar, d.flags, state) & FLAG_ERRORS) return;
         if (tid == 0) *d.rebuild = 0u;
         for_each_particle(bar, n, dyn, [&](int i) { sweep_b_one<DIM, 1, false, AHEAD>(d, g, ph, dt, i); });
-        if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
+        if (grid_sync(bar, d.flags, state) & FLAG_ERRORS) return;
         for_each_particle(bar, n, dyn, [&](int i) { sweep_a_one<DIM, false, AHEAD>(d, g, ph, d.drho_stage, 0, true, d.velq, i); });
         mixed_pass<DIM, false>(d, g, ph, d.drho_stage, d.velq, tid >> 5, stride >> 5, (int)threadIdx.x & 31);
-        if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
+        if (grid_sync(bar, d.flags, state) & FLAG_ERRORS) return;
         for_each_particle(bar, n, dyn, [&](int i) { sweep_b_one<DIM, 2, false, AHEAD>(d, g, ph, dt, i); });
-        if (grid_sync(bar, d.flags, gen) & FLAG_ERRORS) return;
+        if (grid_sync(bar, d.flags, state) & FLAG_ERRORS) return;
     }
 }
 

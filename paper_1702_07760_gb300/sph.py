@@ -444,7 +444,10 @@ class Simulation:
     def neighbours(self):
         L = load()
         start = np.zeros(self.n + 1, np.int64)
-        L.sph_neighbours(self._h, start.ctypes.data_as(C.POINTER(C.c_int64)), None, 0)
+        # the first call gives the row starts (and SPH_EINVAL for want of room)
+        r = L.sph_neighbours(self._h, start.ctypes.data_as(C.POINTER(C.c_int64)), None, 0)
+        if r < 0 and ERRORS.get(int(r)) != "SPH_EINVAL":
+            _check(int(r))
         cap = int(start[-1])
         lst = np.zeros(max(cap, 1), np.int32)
         r = L.sph_neighbours(self._h, start.ctypes.data_as(C.POINTER(C.c_int64)),
