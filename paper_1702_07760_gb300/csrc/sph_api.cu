@@ -63,13 +63,6 @@ struct PendingTiming {
 // (2-D), 193 k 173 against 160 (3-D): the line lies where the 2-D curves cross.
 constexpr int AHEAD_PER_SM = 640;
 
-// Particles an SM above which a sweep is launched while the one before it ends.
-// The dependent launch costs a fixed few us a sweep and fills the end of the sweep before.
-// 20 steps with it against without (us, GB300): 116 k particles 2946 against 2642, 140 k 3147
-// against 2932 (3-D), 105 k 1175 against 1085 (2-D); 238 k 4075 against 4068, 375 k 5305 against
-// 5342, 657 k 8469 against 8514 (3-D).
-constexpr int OVERLAP_PER_SM = 1536;
-
 // Steps in one graph of a small input.
 constexpr int STEPS_PER_GRAPH = 8;
 
@@ -213,22 +206,6 @@ struct sph_sim {
         nvtxRangePop();
     }
 
-    // A sweep launched while the sweep before it may still run (overlap: the
-    // launch before in the stream is a sweep; the kernel waits for it).
-    template <class... P, class... A>
-    void launch_sweep(void (*fn)(P...), int nblocks, int threads, bool overlap, A... args) {
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(nblocks);
-        cfg.blockDim = dim3(threads);
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = overlap && !timing && n > OVERLAP_PER_SM * sms ? 1 : 0;
-        cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
-    }
-
     void collect_timing() {
         for (auto &p : pending) {
             float ms = 0.f;
@@ -320,12 +297,12 @@ void sph_sim::enqueue_eval(int stage, const float *drho_in, double dt)
             using Fn = void (*)(Dev, Grid, Phys, const float *, int, float4 *);
             static const Fn fn[2][2] = {{k_sweep_a<2, false>, k_sweep_a<2, true>},
                                         {k_sweep_a<3, false>, k_sweep_a<3, true>}};
-            launch_sweep(fn[dim - 2][ahead], blocks(n, ta), ta, false, d, grid, phys, drho_in, stage1, vel_s);
+            fn[dim - 2][ahead]<<<blocks(n, ta), ta, 0, stream>>>(d, grid, phys, drho_in, stage1, vel_s);
         } else {
             // warps for the mixed particles: up to eight blocks of eight per SM
             const int mb = std::max(1, std::min(blocks(n), 8 * std::max(sms, 1)));
-            launch_sweep(dim == 2 ? k_sweep_a2<2> : k_sweep_a2<3>, mb + blocks(n), 256, true, d, grid, phys, drho_in,
-                         vel_s, mb);
+            if (dim == 2) k_sweep_a2<2><<<mb + blocks(n), 256, 0, stream>>>(d, grid, phys, drho_in, vel_s, mb);
+            else k_sweep_a2<3><<<mb + blocks(n), 256, 0, stream>>>(d, grid, phys, drho_in, vel_s, mb);
         }
     });
     launch(KI_SWEEP_B, [&] {
@@ -336,7 +313,7 @@ void sph_sim::enqueue_eval(int stage, const float *drho_in, double dt)
              {k_sweep_b<2, 2, false>, k_sweep_b<2, 2, true>}},
             {{k_sweep_b<3, 0, false>, k_sweep_b<3, 0, true>}, {k_sweep_b<3, 1, false>, k_sweep_b<3, 1, true>},
              {k_sweep_b<3, 2, false>, k_sweep_b<3, 2, true>}}};
-        launch_sweep(fn[dim - 2][stage][ahead], blocks(n, tb), tb, true, d, grid, phys, dt);
+        fn[dim - 2][stage][ahead]<<<blocks(n, tb), tb, 0, stream>>>(d, grid, phys, dt);
     });
 }
 

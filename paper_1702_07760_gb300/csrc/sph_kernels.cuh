@@ -1443,29 +1443,12 @@ static __global__ void __launch_bounds__(LIST_THREADS, 1024 / LIST_THREADS) k_bu
 // 45 736 42.7 instead of 44.1, of 96 148 the same.
 constexpr int AHEAD_THREADS = 64, AHEAD_BLOCKS = 6;
 
-// Launches of the sweeps overlap: a sweep is started while the one before it
-// still runs (programmatic dependent launch) and waits here for its results.
-// Each sweep lets the next one start at once; the wait is for the whole grid before,
-// which itself has waited for the one before it.  Used above OVERLAP_PER_SM
-// particles an SM, where it fills the ends of the sweeps (656 600 particles, 20
-// steps 8.51 -> 8.46 ms); smaller inputs were slower with it (9 380 particles 37.7 ->
-// 43.8 us a step, 116 424 132 -> 147).
-// Takes and returns the thread's index: what is read through it, read-only loads
-// included, cannot move above the wait.
-__device__ __forceinline__ int wait_for_launch_before(int i)
-{
-    asm volatile("griddepcontrol.launch_dependents;");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("" : "+r"(i));
-    return i;
-}
-
 template <int DIM, bool AHEAD>
 static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_A_THREADS,
                                          AHEAD ? AHEAD_BLOCKS : 1280 / SPH_SWEEP_A_THREADS)
     k_sweep_a(Dev d, Grid g, Phys ph, const float *__restrict__ drho_in, int stage1, float4 *vel_s)
 {
-    const int i = wait_for_launch_before(blockIdx.x * blockDim.x + threadIdx.x);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d.n) return;
     const int renorm = renorm_now(d, ph, stage1);
     // the lists built for this step are in place; the corrector decides the next build
@@ -1498,13 +1481,12 @@ template <int DIM>
 static __global__ void __launch_bounds__(256) k_sweep_a2(Dev d, Grid g, Phys ph, const float *__restrict__ drho_in,
                                                   float4 *vel_s, int mixed_blocks)
 {
-    const int t = wait_for_launch_before(blockIdx.x * blockDim.x + threadIdx.x);
     if ((int)blockIdx.x < mixed_blocks) {
-        mixed_pass<DIM, true>(d, g, ph, drho_in, vel_s, t >> 5, (int)(mixed_blocks * blockDim.x) >> 5,
-                              (int)threadIdx.x & 31);
+        mixed_pass<DIM, true>(d, g, ph, drho_in, vel_s, (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                              (int)(mixed_blocks * blockDim.x) >> 5, (int)threadIdx.x & 31);
         return;
     }
-    const int i = t - mixed_blocks * (int)blockDim.x;
+    const int i = (int)(blockIdx.x - mixed_blocks) * blockDim.x + threadIdx.x;
     if (i >= d.n) return;
     sweep_a_one<DIM, true>(d, g, ph, drho_in, 0, true, vel_s, i);
 }
@@ -1519,7 +1501,7 @@ static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_B_THR
                                          AHEAD ? AHEAD_BLOCKS : 1024 / SPH_SWEEP_B_THREADS)
     k_sweep_b(Dev d, Grid g, Phys ph, double dt)
 {
-    const int i = wait_for_launch_before(blockIdx.x * blockDim.x + threadIdx.x);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= d.n) return;
     sweep_b_one<DIM, STAGE, true, AHEAD>(d, g, ph, dt, i);
 }
