@@ -676,9 +676,9 @@ def run_ours(args, ws, rank, local):
 
     # per replayed step: the rebuild condition, 2 sweep_a, 2 sweep_b (with the predictor /
     # corrector); per list build in the timed steps: count reset, hash, 3 scan, scatter, rank,
-    # gather, list (the body of the graph's conditional node; up to 640 particles an SM the whole
+    # gather, list (the body of the graph's conditional node; up to 1536 particles an SM the whole
     # rebuild is the step's first kernel instead of the condition)
-    small = w.n <= 640 * torch.cuda.get_device_properties(0).multi_processor_count
+    small = w.n <= 1536 * torch.cuda.get_device_properties(0).multi_processor_count
     launches = 5 * args.steps + (0 if small else 9 * builds_timed)
     line = {
         "metric": "particle-steps/s", "value": value, "unit": "particle-steps/s", "n_gpus": ws,

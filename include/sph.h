@@ -246,7 +246,7 @@ int sph_step(sph_handle h, double dt);
 
 /* nsteps steps of size dt, then waits for the stream and reports any device
  * error.  With graph != 0 the steps are replayed from a CUDA graph captured
- * once per dt.  Up to 640 particles per SM a graph step is five kernels, the
+ * once per dt.  Up to 1 536 particles per SM a graph step is five kernels, the
  * first a cooperative one that rebuilds the lists when the device rebuild flag
  * is set and returns at once otherwise, and runs of eight steps and more
  * replay eight to a graph.  Above that a one-thread kernel copies the flag
@@ -254,8 +254,9 @@ int sph_step(sph_handle h, double dt);
  * chain, so steps without a list build launch five kernels instead of
  * thirteen.  The eager form (graph == 0) launches the same kernels, the
  * cell-list ones returning at once without a build; all forms compute the
- * same bits.
- * The cooperative rebuild (up to 640 particles per SM: here, in sph_step,
+ * same bits.  Above 512 particles per SM a build that is certain (a new state or
+ * step size, a forced build, rebuild_every of 1 to 7) is always the chain.
+ * The cooperative rebuild (here, in sph_step and, up to 512 particles per SM, in
  * sph_build_cells, sph_eval_rates, the queries of neighbours and pairs and the
  * surrogate's calls) waits at grid-wide barriers, each for one second at most.
  * When one gives up, what is queued behind it returns at once without
@@ -307,8 +308,8 @@ int sph_sync(sph_handle h);
 
 /* Test support for the barrier time-out (no counterpart in the paper): puts
  * the handle's grid barrier in a state that no arrival completes, so that the
- * next launch that uses it (sph_run_persistent, or up to 640 particles per SM
- * a list build) waits out its one-second limit in every block and the call
+ * next launch that uses it (sph_run_persistent, or a cooperative rebuild, see
+ * sph_run) waits out its one-second limit in every block and the call
  * that waits for it returns SPH_ETIMEOUT, after which the barrier is reset and
  * runs work again. */
 int sph_test_stall_barrier(sph_handle h);

@@ -54,16 +54,34 @@ struct PendingTiming {
 };
 
 // Particles an SM up to which the sweeps run in blocks of 64 threads and load
-// their neighbours' records a chunk ahead of use.  Small inputs are bound by
+// their neighbours' records a chunk ahead of use (2-D, 3-D).  Small inputs are bound by
 // the latency of a particle's chain of gathers, and blocks of 256 leave SMs idle;
 // large ones by issue and the L1 data pipe, where fewer registers and more warps are
-// better.  A step with the small form against the other (us, GB300, 2-D / 3-D):
-// 9 k particles 32.7 / 96.5 (7 k) against 36.5 / 125.3, 45 k 38.5 against 42.8, 97 k
-// 113.7 against 121.4 (3-D), 140 k 137.8 against 139.4 (3-D), 150 k 58.9 against 54.9
-// (2-D), 193 k 173 against 160 (3-D): the line lies where the 2-D curves cross.
-constexpr int AHEAD_PER_SM = 640;
+// better.  384 threads of that form fit an SM, so its time jumps at each whole wave of 384
+// particles an SM; the lines lie at the last whole wave that beats the large form.  20 steps
+// with it against without, either with the one-kernel rebuild (us, GB300): 2-D, 381 particles an SM
+// 664 against 769, 413 838 against 764, 518 910 against 820; 3-D, 421 (the second wave begun) 1883
+// against 2170, 752 2515 against 2592, 788 2632 against 2607.
+constexpr int AHEAD_PER_SM[2] = {384, 768};
 
-// Steps in one graph of a small input.
+// Particles an SM up to which a step's cell-list chain is one cooperative kernel, and up to
+// which it is also where a build is certain.  Its 512 threads an SM build lists as fast as the
+// chain of kernels while each has one particle (511 an SM, a forced build in 2-D 77 us against
+// 82, in 3-D 149 against 157) and slower beyond (534 an SM in 3-D 170 against 162, 611 209 against
+// 167), but a step without a build saves the conditional node and its launches, some 10 us: 20
+// steps of a stirred tank, which builds every ten steps (3-D) to fifteen (2-D), with it against
+// without: 3-D, 611 an SM 2502 against 2598, 1266 3536 against 3598, 1485 3832 against 3909, 1705 4402
+// against 4358, 2178 5141 against 5044; 2-D, 615 an SM 908 against 1063, 1618 1439 against 1621, 4380
+// 3707 against 3847.  Above the second line a build that the host asks for (a new state or step size)
+// is made by the chain: a loaded state and one step of 611 particles an SM in 3-D 269 us against 297.
+constexpr int ONE_KERNEL_PER_SM = 1536, ONE_KERNEL_BUILD_PER_SM = 512;
+// A fixed cadence (rebuild_every) of fewer steps than this counts as certain.
+constexpr int ONE_KERNEL_CADENCE = 8;
+
+// Steps in one graph of a small input.  200 steps of one step size as graphs of 1, 4, 8 and 16
+// (us, GB300): 9 380 particles 5953, 5465, 5368, 5344; 46 556 6965, 6664, 6516, 6591 (2-D); 72 576
+// 20 169, 19 914, 19 775, 19 764 (3-D).  With a new step size at every call of 8 steps, which
+// captures the graph anew, 329, 358, 410, 333 (9 380).
 constexpr int STEPS_PER_GRAPH = 8;
 
 // Block sizes the persistent kernel is compiled for.  Each size has two
@@ -147,8 +165,8 @@ struct sph_sim {
     int64_t t_launches[KI_COUNT] = {};
     double t_ms[KI_COUNT] = {};
     // per-launch graph of one step, replayed while dt matches
-    // (small inputs: also of several steps)
-    cudaGraphExec_t gexec = nullptr, gexec8 = nullptr;
+    // (small inputs: also of several steps, and of one whose build is due)
+    cudaGraphExec_t gexec = nullptr, gexec8 = nullptr, gexec_due = nullptr;
     double gdt = 0.0;
     // persistent form: launch shape and its graph
     int pbs = 256, pgrid = 0;             // block size, grid blocks (0: as many as fit)
@@ -222,15 +240,28 @@ struct sph_sim {
     int blocks(int work, int threads = 256) const { return (work + threads - 1) / threads; }
     int sms = 0;  // multiprocessors of the device
 
-    // small inputs rebuild in one cooperative kernel of at most two blocks an SM (the per-kernel
-    // timing keeps the chain)
-    bool one_kernel_rebuild() const { return !timing && n <= AHEAD_PER_SM * sms; }
+    // Whether the lists are built by one cooperative kernel of at most two blocks an SM (the
+    // per-kernel timing keeps the chain): where a build is certain, and in steps that may build.
+    bool one_kernel_build() const { return !timing && n <= ONE_KERNEL_BUILD_PER_SM * sms; }
+    bool one_kernel_steps() const {
+        const bool often = P.rebuild_every > 0 && P.rebuild_every < ONE_KERNEL_CADENCE;
+        return often ? one_kernel_build() : !timing && n <= ONE_KERNEL_PER_SM * sms;
+    }
+    // Raises the device flag `rebuild`; build_due notes it for the choice above (only for
+    // that: every build looks at the device flag).
+    bool build_due = false;
+    cudaError_t raise_rebuild() {
+        build_due = true;
+        return cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream);
+    }
     void enqueue_build_cells(bool force);
+    void enqueue_build_chain();
+    void drop_step_graphs();
     void enqueue_load(const double *x, const double *u, const double *rho, double check_dt);
     int enqueue_read(int kind, bool integer, void *out, size_t bytes, size_t staging_offset);
     void enqueue_eval(int stage, const float *drho_in, double dt);
     void enqueue_step(double dt);
-    int capture_step_graph(double dt, int steps, cudaGraphExec_t *out);
+    int capture_step_graph(double dt, int steps, bool chain, cudaGraphExec_t *out);
     int enqueue_set_state(const double *x, const double *u, const double *rho);
     int enqueue_run(double dt, int64_t nsteps, bool graph);
     int enqueue_read_state(double *x, double *u, double *rho);
@@ -245,10 +276,8 @@ struct sph_sim {
 // launch sequence serves every step of a captured graph.
 void sph_sim::enqueue_build_cells(bool force)
 {
-    Dev &s = buf[0];
-    Dev &t = buf[1];
-    if (force) cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream);
-    if (one_kernel_rebuild()) {
+    if (force) raise_rebuild();
+    if (build_due ? one_kernel_build() : one_kernel_steps()) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(std::min(blocks(n), 2 * sms));
         cfg.blockDim = dim3(256);
@@ -258,9 +287,16 @@ void sph_sim::enqueue_build_cells(bool force)
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaLaunchKernelEx(&cfg, dim == 2 ? k_rebuild<2> : k_rebuild<3>, s, t, grid, phys, sort, bar);
+        cudaLaunchKernelEx(&cfg, dim == 2 ? k_rebuild<2> : k_rebuild<3>, buf[0], buf[1], grid, phys, sort, bar);
         return;
     }
+    enqueue_build_chain();
+}
+
+void sph_sim::enqueue_build_chain()
+{
+    Dev &s = buf[0];
+    Dev &t = buf[1];
     launch(KI_MEMSET, [&] { k_zero<<<blocks(ncell), 256, 0, stream>>>(sort.count, ncell, rebuild); });
     launch(KI_HASH, [&] {
         if (dim == 2) k_hash<2><<<blocks(n), 256, 0, stream>>>(s, grid, sort);
@@ -290,7 +326,8 @@ void sph_sim::enqueue_eval(int stage, const float *drho_in, double dt)
     Dev &d = buf[0];
     float4 *vel_s = stage == 2 ? d.velq : d.velp;
     const int stage1 = stage != 2;
-    const bool ahead = n <= AHEAD_PER_SM * sms;
+    const bool ahead = n <= AHEAD_PER_SM[dim - 2] * sms;
+    if (stage1) build_due = false;   // sweep A lowers the flag
     launch(KI_SWEEP_A, [&] {
         if (stage1) {
             const int ta = ahead ? AHEAD_THREADS : SPH_SWEEP_A_THREADS;
@@ -329,15 +366,15 @@ namespace {
 __global__ void k_rebuild_cond(cudaGraphConditionalHandle h, const unsigned *rebuild);
 }  // namespace
 
-// The replayed step as a graph.  Small inputs (one_kernel_rebuild): `steps`
-// steps of five kernels, the first the rebuild in one kernel.  Otherwise one
+// The replayed step as a graph.  Without `chain` (one_kernel_steps): `steps`
+// steps of five kernels, the first the rebuild in one kernel.  With it one
 // step: a one-thread kernel reads the rebuild flag into the condition of an IF
 // node whose body is the cell-list chain, then the four sweeps.  On steps
 // without a rebuild the chain is not launched at all (its kernels would return
 // at once, but nine launches of n/256 blocks still cost several microseconds
 // each).  The body's kernels keep their own flag test, so the graph and the
 // eager sequence compute the same.
-int sph_sim::capture_step_graph(double dt, int steps, cudaGraphExec_t *out)
+int sph_sim::capture_step_graph(double dt, int steps, bool chain, cudaGraphExec_t *out)
 {
     cudaGraph_t g = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -357,7 +394,7 @@ int sph_sim::capture_step_graph(double dt, int steps, cudaGraphExec_t *out)
         cudaGraphDestroy(g);
         return fail(SPH_ECUDA, std::string(what) + ": " + cudaGetErrorString(err));
     };
-    if (one_kernel_rebuild()) {
+    if (!chain) {
         // no conditional node: the rebuild kernel returns at once on steps without a build
         if ((e = cudaStreamBeginCaptureToGraph(stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
             cudaSuccess)
@@ -389,7 +426,7 @@ int sph_sim::capture_step_graph(double dt, int steps, cudaGraphExec_t *out)
     if ((e = cudaStreamBeginCaptureToGraph(stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal)) !=
         cudaSuccess)
         return bail("graph capture", e);
-    enqueue_build_cells(false);
+    enqueue_build_chain();
     if ((e = cudaStreamEndCapture(stream, &body)) != cudaSuccess) return bail("graph capture", e);
     if ((e = cudaStreamBeginCaptureToGraph(stream, g, &cond, nullptr, 1, cudaStreamCaptureModeThreadLocal)) !=
         cudaSuccess)
@@ -402,6 +439,14 @@ int sph_sim::capture_step_graph(double dt, int steps, cudaGraphExec_t *out)
     if (*out) cudaGraphExecDestroy(*out);
     *out = exec;
     return SPH_OK;
+}
+
+void sph_sim::drop_step_graphs()
+{
+    for (cudaGraphExec_t *g : {&gexec, &gexec8, &gexec_due}) {
+        if (*g) cudaGraphExecDestroy(*g);
+        *g = nullptr;
+    }
 }
 
 // Grid and kernel build of a persistent launch of grid_req blocks of bs
@@ -460,7 +505,7 @@ int sph_sim::check_flags()
         // the steps that the device has made
         long long done = 0;
         CU(cudaMemsetAsync(bar, 0, sizeof(GridBarrier), stream));
-        CU(cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream));
+        CU(raise_rebuild());
         CU(cudaMemcpyAsync(&done, dstep, sizeof(done), cudaMemcpyDeviceToHost, stream));
         CU(cudaStreamSynchronize(stream));
         last_dt = 0.0;
@@ -1218,7 +1263,11 @@ SimView sim_view(sph_sim *s)
     return v;
 }
 
-void sim_evaluated(sph_sim *s) { s->evaluated = true; }
+void sim_evaluated(sph_sim *s)
+{
+    s->evaluated = true;
+    s->build_due = false;
+}
 
 void sim_build_lists(sph_sim *s)
 {
@@ -1232,7 +1281,7 @@ int sim_moved(sph_sim *s, int64_t steps, double elapsed)
     if (s->n > 0) {
         k_add_step<<<1, 32, 0, s->stream>>>(s->D(), s->dstep, (long long)steps, s->clock, elapsed);
         CU(cudaGetLastError());
-        CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
+        CU(s->raise_rebuild());
     }
     s->step += steps;
     return SPH_OK;
@@ -1260,7 +1309,7 @@ int sim_load_device(sph_sim *s, const double *x, const double *u, const double *
     if (s->n == 0) return SPH_OK;
     s->enqueue_load(x, u, rho, 0.0);
     CU(cudaGetLastError());
-    CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
+    CU(s->raise_rebuild());
     return SPH_OK;
 }
 
@@ -1385,7 +1434,7 @@ int sph_sim::enqueue_set_state(const double *x, const double *u, const double *r
     const double check_dt = P.rebuild_every == 0 ? last_dt : 0.0;
     enqueue_load(dx, du, dr, check_dt);
     CU(cudaGetLastError());
-    if (!(check_dt > 0)) CU(cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream));
+    if (!(check_dt > 0)) CU(raise_rebuild());
     return SPH_OK;
 }
 
@@ -1513,7 +1562,7 @@ int sph_perturb_state(sph_handle s, double sigma_u, double sigma_rho, uint64_t s
     else k_perturb<3><<<s->blocks(s->n), 256, 0, s->stream>>>(s->D(), sigma_u, sigma_rho, seed);
     CU(cudaGetLastError());
     // the stage records derive from the state: rebuilt with the lists
-    CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
+    CU(s->raise_rebuild());
     return SPH_OK;
 }
 
@@ -1543,7 +1592,7 @@ int sph_set_dt_scales(sph_handle s, const double *scales)
     for (int q = 0; q < s->ninst; ++q) s->hinst[q].dt_scale = scales[q];
     CU(cudaMemcpyAsync(s->dinst, s->hinst.data(), sizeof(Inst) * s->ninst, cudaMemcpyHostToDevice, s->stream));
     // the rebuild test looks half a step ahead with the previous step size
-    CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
+    CU(s->raise_rebuild());
     CU(cudaStreamSynchronize(s->stream));
     return SPH_OK;
 }
@@ -1575,7 +1624,7 @@ int sph_step(sph_handle s, double dt)
     if (!(dt > 0) || !std::isfinite(dt)) return fail(SPH_EINVAL, "dt must be positive and finite");
     if (s->n > 0) {
         // the rebuild test looks half a step ahead with the previous dt
-        if (dt != s->last_dt) CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
+        if (dt != s->last_dt) CU(s->raise_rebuild());
         s->last_dt = dt;
         s->enqueue_step(dt);
         CU(cudaGetLastError());
@@ -1604,19 +1653,35 @@ int sph_run(sph_handle s, double dt, int64_t nsteps, int graph)
 int sph_sim::enqueue_run(double dt, int64_t nsteps, bool graph)
 {
     const bool use_graph = graph && !timing;
-    if (dt != last_dt) CU(cudaMemsetAsync(rebuild, 0xff, sizeof(unsigned), stream));
+    if (dt != last_dt) CU(raise_rebuild());
     last_dt = dt;
     if (use_graph) {
-        if (gdt != dt) {
-            if (gexec) cudaGraphExecDestroy(gexec);
-            if (gexec8) cudaGraphExecDestroy(gexec8);
-            gexec = gexec8 = nullptr;
+        const bool new_dt = gdt != dt, one = one_kernel_steps();
+        if (new_dt) {
+            drop_step_graphs();
             gdt = dt;
         }
         int64_t k = 0;
-        if (one_kernel_rebuild() && nsteps >= STEPS_PER_GRAPH) {
+        if (nsteps > 0 && build_due && one && !one_kernel_build()) {
+            // a step whose build is due, and faster as the chain: a graph of its own, but for
+            // a new step size, which may not come again
+            if (new_dt) {
+                enqueue_step(dt);
+                CU(cudaGetLastError());
+            } else {
+                if (!gexec_due) {
+                    const int rc = capture_step_graph(dt, 1, true, &gexec_due);
+                    if (rc != SPH_OK) return rc;
+                }
+                CU(cudaGraphLaunch(gexec_due, stream));
+            }
+            step += 1;
+            k = 1;
+        }
+        if (nsteps > 0) build_due = false;
+        if (one && nsteps - k >= STEPS_PER_GRAPH) {
             if (!gexec8) {
-                const int rc = capture_step_graph(dt, STEPS_PER_GRAPH, &gexec8);
+                const int rc = capture_step_graph(dt, STEPS_PER_GRAPH, false, &gexec8);
                 if (rc != SPH_OK) return rc;
             }
             for (; k + STEPS_PER_GRAPH <= nsteps; k += STEPS_PER_GRAPH) {
@@ -1625,7 +1690,7 @@ int sph_sim::enqueue_run(double dt, int64_t nsteps, bool graph)
             }
         }
         if (k < nsteps && !gexec) {
-            const int rc = capture_step_graph(dt, 1, &gexec);
+            const int rc = capture_step_graph(dt, 1, !one, &gexec);
             if (rc != SPH_OK) return rc;
         }
         for (; k < nsteps; ++k) {
@@ -1653,8 +1718,9 @@ int sph_run_persistent(sph_handle s, double dt, int64_t nsteps, int graph)
         s->step += nsteps;
         return SPH_OK;
     }
-    if (dt != s->last_dt) CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
+    if (dt != s->last_dt) CU(s->raise_rebuild());
     s->last_dt = dt;
+    s->build_due = false;   // the kernel builds by itself
     const int shape = (s->pbs * 100000 + s->pgrid) * 2 + s->pdyn;
     if (graph && !s->timing) {
         if (!s->pexec || s->pdt != dt || s->psteps != nsteps || s->pshape != shape) {
@@ -1795,7 +1861,7 @@ int sph_autotune(sph_handle s, double dt, int trial_steps, int *best_block, int 
     // rebuilds the lists)
     int rc2 = sph_set_state(s, x.data(), u.data(), rho.data());
     CU(cudaMemcpyAsync(s->clock, clock, sizeof(clock), cudaMemcpyHostToDevice, s->stream));
-    CU(cudaMemsetAsync(s->rebuild, 0xff, sizeof(unsigned), s->stream));
+    CU(s->raise_rebuild());
     CU(cudaMemcpyAsync(s->dstep, &dstep, sizeof(dstep), cudaMemcpyHostToDevice, s->stream));
     CU(cudaMemcpyAsync(s->dbuilds, &dbuilds, sizeof(dbuilds), cudaMemcpyHostToDevice, s->stream));
     CU(cudaStreamSynchronize(s->stream));
@@ -2104,8 +2170,7 @@ void sph_destroy(sph_handle s)
     if (s->ext && s->ext_free) s->ext_free(s->ext);
     s->collect_timing();
     for (auto e : s->free_events) cudaEventDestroy(e);
-    if (s->gexec) cudaGraphExecDestroy(s->gexec);
-    if (s->gexec8) cudaGraphExecDestroy(s->gexec8);
+    s->drop_step_graphs();
     if (s->pexec) cudaGraphExecDestroy(s->pexec);
     for (void *p : s->allocs) cudaFree(p);
     if (s->own_stream) cudaStreamDestroy(s->stream);

@@ -1191,8 +1191,8 @@ __device__ __forceinline__ void prefetch_epilogue(const Dev &d, int k)
 // (Eq. ct_dist_2).  grad_i W_ij = cF t^3 r_ij with t = 1 - q/2; the common
 // factor cF is applied once per particle.
 // STAGE 0: rates only; 1: then the predictor; 2: then the corrector.
-// The launches of small inputs (AHEAD, not in the persistent kernel) follow the
-// one-kernel rebuild and do nothing when its barrier gave up.
+// The launches (NC: not the persistent kernel) may follow the one-kernel rebuild and do
+// nothing when its barrier gave up.
 template <int DIM, int STAGE, bool NC, bool AHEAD = false>
 __device__ __forceinline__ void sweep_b_one(const Dev &d, const Grid &g, const Phys &ph, double dt, int i)
 {
@@ -1211,7 +1211,7 @@ __device__ __forceinline__ void sweep_b_one(const Dev &d, const Grid &g, const P
     // list) add exact zeros while those are at rest: u_ij = 0 in the
     // continuity term, and the acceleration of a boundary particle is not used
     const int n = d.n, cnt = ld<NC>(d.walls_moving) ? d.ncnt[i] : d.nfcnt[i];
-    if (NC && AHEAD && stopped(d)) return;
+    if (NC && stopped(d)) return;
     if (STAGE != 0) prefetch_epilogue<DIM, STAGE>(d, i);
     // per-phase constants of the pair terms as registers (selected per pair):
     // m_j P_i / rho_i^2 for a water and an oil neighbour, and the viscous factors
@@ -1452,7 +1452,7 @@ static __global__ void __launch_bounds__(AHEAD ? AHEAD_THREADS : SPH_SWEEP_A_THR
     if (i >= d.n) return;
     const int renorm = renorm_now(d, ph, stage1);
     // the lists built for this step are in place; the corrector decides the next build
-    if (stage1 && i == 0 && !(AHEAD && stopped(d))) {
+    if (stage1 && i == 0 && !stopped(d)) {
         *d.rebuild = 0u;
         d.clock[0] += d.clock[1];
         d.clock[1] = 0.0;

@@ -6,6 +6,8 @@ persistent kernel's two builds (up to 512 particles an SM, 77 824, and above).
 
 All of them do the same arithmetic per particle in the same order, so every
 form gives the same bits.
+
+(Where the lines lie by now: test_builds_asked_for_and_builds_that_come_up.)
 """
 import numpy as np
 import pytest
@@ -126,3 +128,57 @@ def test_large_inputs_give_the_same_bits_in_every_form(sphmod, shape):
         s.timing(False)
     for f in ("acc", "drho", "pressure", "rho_eval", "tensor"):
         assert np.array_equal(graph.read(f), timed.read(f)), f
+
+
+# The lines as they stand, in particles an SM (x 152 SMs): blocks that load ahead up to 384 in
+# 2-D (58 368; 208 x 280 = 58 240 and 209 x 280 = 58 520 particles) and 768 in 3-D (116 736; 36 x 54 x 60 =
+# 116 640 and 37 x 54 x 60 = 119 880); a certain build in one kernel up to 512 (77 824; 272 x 286 and
+# 273 x 286), a step's up to 1 536 (233 472; 48 x 64 x 76 = 233 472 and 49 x 64 x 76 = 238 336).
+@pytest.mark.parametrize("shape", [(202, 274), (203, 274), (266, 280), (267, 280),
+                                   (30, 48, 54), (31, 48, 54), (42, 58, 70), (43, 58, 70)])
+def test_builds_asked_for_and_builds_that_come_up(sphmod, shape):
+    """Builds that the host asks for (a first run, a new state, a new step size, a forced build)
+    between builds that a step finds due, through every form: the same bits and as many builds."""
+    import torch
+    w = WL.drop_tank(len(shape), shape, drop_d_dx=min(shape) / 3, seed=sum(shape), perturb=True)
+    dt = WL.stable_dt(w.params)
+    state = [torch.tensor(a, dtype=torch.float64, device="cuda") for a in (w.x, w.u, w.rho)]
+
+    def go(s, run):
+        run(s, dt, 9)
+        s.load_snapshot(*[a.data_ptr() for a in state])
+        run(s, dt, 1)
+        run(s, dt, 10)
+        run(s, 0.9 * dt, 3)
+        s.build_cells()
+        run(s, 0.9 * dt, 8)
+        s.eval_rates()
+        run(s, 0.9 * dt, 2)
+        s.set_state(w.x, w.u, w.rho)
+        run(s, 0.9 * dt, 2)
+        return s
+
+    new = lambda: sphmod.Simulation.from_workload(w)  # noqa: E731
+    graph = go(new(), lambda s, d, k: s.run(d, k))
+    _same(graph, go(new(), lambda s, d, k: s.run(d, k, graph=False)))
+    _same(graph, go(new(), lambda s, d, k: s.run_persistent(d, k)))
+    timed = new()
+    timed.timing(True)
+    _same(graph, go(timed, lambda s, d, k: s.run(d, k)))
+
+
+@pytest.mark.parametrize("every", [1, 3, 8])
+@pytest.mark.parametrize("shape", [(40, 40), (300, 300)])
+def test_fixed_cadences(sphmod, shape, every):
+    """Every, every third and every eighth step builds, below and above 512 particles an SM."""
+    w = WL.drop_tank(2, shape, drop_d_dx=min(shape) / 3, seed=every, perturb=True)
+    w.params["rebuild_every"] = every
+    dt = 0.25 * WL.stable_dt(w.params)   # a fixed cadence reports a motion beyond the skin
+    graph, eager, persistent = (sphmod.Simulation.from_workload(w) for _ in range(3))
+    graph.run(dt, 3)
+    graph.run(dt, 17)
+    eager.run(dt, 20, graph=False)
+    persistent.run_persistent(dt, 20)
+    assert graph.list_builds >= 20 // every
+    for s in (eager, persistent):
+        _same(graph, s)
