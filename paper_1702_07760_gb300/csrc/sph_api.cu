@@ -7,6 +7,8 @@
 #include "sph_internal.h"
 #include "sph_kernels.cuh"
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -114,6 +116,34 @@ PersistFn persist_fn(int dim, int bs, bool wide)
 }
 
 }  // namespace
+
+// A driver function of the given version, looked up through the runtime; NULL when there is none.
+template <class F>
+F driver_fn(const char *name, int version)
+{
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion(name, &p, version, cudaEnableDefault, &q) != cudaSuccess) cudaGetLastError();
+    return q == cudaDriverEntryPointSuccess ? (F)p : nullptr;
+}
+
+// The multiprocessors that kernels on the stream may use: the device's, or those of the green
+// context that the stream was made in.  (A cooperative launch of more blocks than they hold is refused.)
+cudaError_t stream_sms(cudaStream_t st, int *sms)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const auto context_of = driver_fn<PFN_cuStreamGetGreenCtx_v12040>("cuStreamGetGreenCtx", 12040);
+    const auto resource_of = driver_fn<PFN_cuGreenCtxGetDevResource_v12040>("cuGreenCtxGetDevResource", 12040);
+    CUgreenCtx green = nullptr;
+    CUdevResource r{};
+    if (context_of && resource_of && context_of((CUstream)st, &green) == CUDA_SUCCESS && green &&
+        resource_of(green, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && r.sm.smCount > 0)
+        *sms = std::min(*sms, (int)r.sm.smCount);
+    return cudaSuccess;
+}
 
 struct sph_sim {
     sph_params P{};
@@ -238,14 +268,15 @@ struct sph_sim {
     }
 
     int blocks(int work, int threads = 256) const { return (work + threads - 1) / threads; }
-    int sms = 0;  // multiprocessors of the device
+    int sms = 0;          // multiprocessors that the stream's kernels may use
+    int rebuild_fit = 0;  // blocks of the one-kernel rebuild on one of them: two, or what fits
 
-    // Whether the lists are built by one cooperative kernel of at most two blocks an SM (the
+    // Whether the lists are built by one cooperative kernel, all of whose blocks are resident (the
     // per-kernel timing keeps the chain): where a build is certain, and in steps that may build.
-    bool one_kernel_build() const { return !timing && n <= ONE_KERNEL_BUILD_PER_SM * sms; }
+    bool one_kernel_build() const { return !timing && rebuild_fit > 0 && n <= ONE_KERNEL_BUILD_PER_SM * sms; }
     bool one_kernel_steps() const {
         const bool often = P.rebuild_every > 0 && P.rebuild_every < ONE_KERNEL_CADENCE;
-        return often ? one_kernel_build() : !timing && n <= ONE_KERNEL_PER_SM * sms;
+        return often ? one_kernel_build() : !timing && rebuild_fit > 0 && n <= ONE_KERNEL_PER_SM * sms;
     }
     // Raises the device flag `rebuild`; build_due notes it for the choice above (only for
     // that: every build looks at the device flag).
@@ -279,7 +310,7 @@ void sph_sim::enqueue_build_cells(bool force)
     if (force) raise_rebuild();
     if (build_due ? one_kernel_build() : one_kernel_steps()) {
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(std::min(blocks(n), 2 * sms));
+        cfg.gridDim = dim3(std::min(blocks(n), rebuild_fit * sms));
         cfg.blockDim = dim3(256);
         cfg.stream = stream;
         cudaLaunchAttribute attr[1];
@@ -1173,11 +1204,11 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
     if ((e = cudaMemsetAsync(a0.ncnt, 0, sizeof(int) * N, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaMemsetAsync(a0.nfcnt, 0, sizeof(int) * N, st)) != cudaSuccess) return cuda_fail(e);
     if ((e = cudaMemsetAsync(a0.nflag, 0, N, st)) != cudaSuccess) return cuda_fail(e);
-    {
-        int dev = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return cuda_fail(e);
-        if ((e = cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return cuda_fail(e);
-    }
+    if ((e = stream_sms(st, &s->sms)) != cudaSuccess) return cuda_fail(e);
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+             &s->rebuild_fit, dim == 2 ? (const void *)k_rebuild<2> : (const void *)k_rebuild<3>, 256, 0)) != cudaSuccess)
+        return cuda_fail(e);
+    s->rebuild_fit = std::min(s->rebuild_fit, 2);
     {
         // super-cell centres per axis (the FP64 offsets' origins)
         std::vector<double> cen;
@@ -1664,16 +1695,15 @@ int sph_sim::enqueue_run(double dt, int64_t nsteps, bool graph)
         int64_t k = 0;
         if (nsteps > 0 && build_due && one && !one_kernel_build()) {
             // a step whose build is due, and faster as the chain: a graph of its own, but for
-            // a new step size, which may not come again
-            if (new_dt) {
+            // a new step size, which may not come again, and where the conditional node is
+            // refused (streams of green contexts)
+            if (!new_dt && !gexec_due && capture_step_graph(dt, 1, true, &gexec_due) != SPH_OK) cudaGetLastError();
+            if (gexec_due) {
+                CU(cudaGraphLaunch(gexec_due, stream));
+            } else {
+                build_due = true;   // (a capture has cleared it)
                 enqueue_step(dt);
                 CU(cudaGetLastError());
-            } else {
-                if (!gexec_due) {
-                    const int rc = capture_step_graph(dt, 1, true, &gexec_due);
-                    if (rc != SPH_OK) return rc;
-                }
-                CU(cudaGraphLaunch(gexec_due, stream));
             }
             step += 1;
             k = 1;
