@@ -1410,6 +1410,22 @@ int enqueue_train_step(sph_handle h, Surrogate &S, bool update)
     return pack_weights(S, v.stream);
 }
 
+// The step's launches as a graph; NULL where the stream does not allow it (nothing has been
+// launched then).
+cudaGraphExec_t capture_train_step(sph_handle h, Surrogate &S, bool update, cudaStream_t st)
+{
+    cudaGraph_t g = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        const int rc = enqueue_train_step(h, S, update);
+        const cudaError_t e = cudaStreamEndCapture(st, &g);
+        if (!rc && e == cudaSuccess && cudaGraphInstantiate(&exec, g, 0) != cudaSuccess) exec = nullptr;
+        if (g) cudaGraphDestroy(g);
+    }
+    cudaGetLastError();   // a refusal is not an error of the step
+    return exec;
+}
+
 int check_err(Surrogate &S, cudaStream_t st)
 {
     unsigned e = 0;
@@ -1593,23 +1609,16 @@ int sph_surrogate_train_step(sph_handle h, const double *x1, const double *u1, c
         S->args_h->eps_t = (float)(eps * std::sqrt(c2));
     }
     CUR(cudaMemcpyAsync(S->args, S->args_h, sizeof(StepArgs), cudaMemcpyHostToDevice, v0.stream));
-    // the first step of each kind launches kernel by kernel, later ones replay its graph
+    // the first step of each kind launches kernel by kernel, later ones replay its graph, but
+    // where there is none (cudaStreamLegacy cannot be captured)
     cudaGraphExec_t &graph = S->step_graph[update ? 1 : 0];
-    if (S->step_calls[update ? 1 : 0]++ == 0 || v0.timing) {
-        if ((rc = enqueue_train_step(h, *S, update != 0))) return rc;
-    } else {
-        if (!graph) {
-            cudaGraph_t g = nullptr;
-            CUR(cudaStreamBeginCapture(v0.stream, cudaStreamCaptureModeThreadLocal));
-            rc = enqueue_train_step(h, *S, update != 0);
-            cudaError_t ce = cudaStreamEndCapture(v0.stream, &g);
-            if (!rc && ce == cudaSuccess) ce = cudaGraphInstantiate(&graph, g, 0);
-            if (g) cudaGraphDestroy(g);
-            if (rc) return rc;
-            if (ce != cudaSuccess) return set_error(SPH_ECUDA, std::string("training graph: ") + cudaGetErrorString(ce));
-        }
+    if (S->step_calls[update ? 1 : 0]++ > 0 && !v0.timing && !graph)
+        graph = capture_train_step(h, *S, update != 0, v0.stream);
+    if (graph && !v0.timing) {
         CUR(cudaGraphLaunch(graph, v0.stream));
         sim_evaluated(h);
+    } else if ((rc = enqueue_train_step(h, *S, update != 0))) {
+        return rc;
     }
     if (update) S->adam_t = t;
     const SimView v = v0;

@@ -1,12 +1,13 @@
 """Handles on streams of the caller's that are not ordinary ones: of a green context, which
-gives its kernels a part of the multiprocessors."""
+gives its kernels a part of the multiprocessors, and the legacy default stream, which cannot be
+captured into a graph."""
 import ctypes as C
 
 import numpy as np
 import pytest
 
 from paper_1702_07760_gb300 import workloads as WL
-from test_gpu_surrogate import env  # noqa: F401
+from test_gpu_surrogate import _case, env  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -70,3 +71,31 @@ def test_part_of_the_multiprocessors(env, green_stream, shape):  # noqa: F811
     assert s.list_builds == ref.list_builds
     s.close()
     ref.close()
+
+
+@pytest.mark.parametrize("stream", [1, 2])   # cudaStreamLegacy, cudaStreamPerThread
+@pytest.mark.parametrize("dim", [2, 3])
+def test_training_on_default_streams(env, dim, stream):  # noqa: F811
+    """Every step after the first replays a graph where the stream can be captured, and is
+    launched where it cannot: the loss to the order of FP64 sums (1e-10), the gradient to that of
+    FP32 ones (1e-5 of its norm)."""
+    torch, sph = env
+    w, norm, flat = _case(dim, 50 + dim)
+    rng = np.random.Generator(np.random.PCG64(51))
+    free = (w.wall == 0)[:, None]
+    t = [torch.tensor(a, dtype=torch.float64, device="cuda")
+         for a in (w.x + free * rng.normal(0, 1e-6, w.x.shape), w.u + free * rng.normal(0, 1e-2, w.u.shape),
+                   w.rho * (1 + rng.normal(0, 1e-4, w.n)))]
+    torch.cuda.synchronize()
+    s, ref = sph.Simulation.from_workload(w, stream=stream), sph.Simulation.from_workload(w)
+    for h in (s, ref):
+        h.surrogate_init(flat, norm)
+    for _ in range(3):
+        s.surrogate_train_step(*[a.data_ptr() for a in t], lr=1e-3)
+    assert np.abs(s.surrogate_weights() - flat).max() > 1e-3   # three updates were made
+    s.surrogate_init(flat, norm)
+    for _ in range(3):
+        loss, g = s.surrogate_train_step(*[a.data_ptr() for a in t], update=False, want_grad=True)
+        loss1, g1 = ref.surrogate_train_step(*[a.data_ptr() for a in t], update=False, want_grad=True)
+        assert abs(loss - loss1) <= 1e-10 * loss1
+        assert np.linalg.norm(g - g1) <= 1e-5 * np.linalg.norm(g1)
