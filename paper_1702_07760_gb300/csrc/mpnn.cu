@@ -159,7 +159,8 @@ struct Surrogate {
         for (void *p : allocs) cudaFree(p);
         if (loss_h) cudaFreeHost(loss_h);
         drop_graphs();
-        for (cudaEvent_t e : fork) cudaEventDestroy(e);
+        for (cudaEvent_t e : fork)
+            if (e) cudaEventDestroy(e);
         for (cudaEvent_t e : join)
             if (e) cudaEventDestroy(e);
         for (cudaStream_t t : side)
@@ -1044,25 +1045,27 @@ int alloc_surrogate(Surrogate &S)
     return SPH_OK;
 }
 
-// Particles up to which the backward pass keeps a buffer per layer and takes
-// the weight and bias gradients beside the data gradients (9.5 KB a particle);
-// beyond, the layers share one set of buffers and one stream.
-constexpr int SIDE_MAX = 1 << 23;
+// Particles up to which the backward pass keeps a buffer per layer and takes the weight and
+// bias gradients beside the data gradients; beyond, or where that much memory is not there, the
+// layers share one set of buffers and one stream (10.1 against 4.2 KB a particle).  A training step
+// with one set against a set per layer (GB300): 3 220 particles 857 against 583 us, 46 556 1846
+// against 1490, 77 976 5474 against 5177, 193 496 12.18 against 11.95 ms, 335 000 19.91 against 19.78,
+// 656 600 38.91 against 38.77: beyond a million the 5.9 KB a particle buy next to nothing.
+constexpr int SIDE_MAX = 1 << 20;
 
-int alloc_backward(Surrogate &S)
+// The device buffers of the backward pass; all of them or none.
+int alloc_backward_set(Surrogate &S, bool own, float **dS)
 {
-    if (S.dS) return SPH_OK;
-    const size_t P = (size_t)S.npad;
-    const bool own = S.n <= SIDE_MAX;
+    const size_t P = (size_t)S.npad, mark = S.allocs.size();
     int e = 0;
-    e |= dalloc(S, &S.dYf, P * FOUT);
-    e |= dalloc(S, &S.dYb, P * FOUT);
     auto layers = [&](auto *p, int count, size_t width) {
-        for (int k = 0; k < count; ++k) {
+        for (int k = 0; k < count && !e; ++k) {
             if (k == 0 || own) e |= dalloc(S, &p[k], P * width);
             else p[k] = p[0];
         }
     };
+    layers(&S.dYf, 1, FOUT);
+    layers(&S.dYb, 1, FOUT);
     layers(S.dZf, 4, H);
     layers(S.dZb, 4, H);
     layers(S.dA, 2, 2 * H);
@@ -1070,16 +1073,20 @@ int alloc_backward(Surrogate &S)
     layers(S.dh, 3, H);
     layers(S.dhb, 3, H);
     layers(S.dPQ, 2, 2 * H);
-    e |= dalloc(S, &S.sums, SUMS);
-    e |= dalloc(S, &S.args, 1);
-    if (own && !S.side[0]) {
-        S.fork.resize(BWD_LAYERS);
-        for (cudaEvent_t &ev : S.fork) CUR(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-        for (int k = 0; k < 2; ++k) {
-            CUR(cudaStreamCreateWithFlags(&S.side[k], cudaStreamNonBlocking));
-            CUR(cudaEventCreateWithFlags(&S.join[k], cudaEventDisableTiming));
-        }
+    layers(dS, 1, H);
+    if (!e) e = dalloc(S, &S.sums, SUMS);
+    if (!e) e = dalloc(S, &S.args, 1);
+    if (e) {
+        for (; S.allocs.size() > mark; S.allocs.pop_back()) cudaFree(S.allocs.back());
+        cudaGetLastError();   // the refused allocation is not an error of what follows
+        return SPH_ENOMEM;
     }
+    return SPH_OK;
+}
+
+int alloc_backward(Surrogate &S)
+{
+    if (S.dS) return SPH_OK;
     if (!S.loss_h) {
         void *q = nullptr;
         const cudaError_t ce = cudaMallocHost(&q, sizeof(double) + sizeof(StepArgs) + sizeof(float) * S.L.total);
@@ -1088,9 +1095,22 @@ int alloc_backward(Surrogate &S)
         S.args_h = reinterpret_cast<StepArgs *>(S.loss_h + 1);
         S.grad_h = reinterpret_cast<float *>(S.args_h + 1);
     }
-    e |= dalloc(S, &S.dS, P * H);
-    if (e) return SPH_ENOMEM;
+    bool own = S.n <= SIDE_MAX;
+    float *dS = nullptr;
+    int rc = alloc_backward_set(S, own, &dS);
+    if (rc && own) rc = alloc_backward_set(S, own = false, &dS);
+    if (rc) return rc;
+    if (own) {
+        S.fork.resize(BWD_LAYERS, nullptr);
+        for (cudaEvent_t &ev : S.fork)
+            if (!ev) CUR(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        for (cudaEvent_t &ev : S.join)
+            if (!ev) CUR(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        for (cudaStream_t &t : S.side)
+            if (!t) CUR(cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking));
+    }
     CUR(cudaDeviceSynchronize());
+    S.dS = dS;
     return SPH_OK;
 }
 
