@@ -65,3 +65,57 @@ def test_three_dimensions_and_an_uneven_batch(sphmod):
     for _ in range(2):
         for d, q in zip(sim.diagnostics_instances(), ws):
             _check(d, q)
+
+
+def _state_of(sim, w):
+    return WL.Workload(w.name, w.params, sim.read("pos"), sim.read("vel"), sim.read("rho"), w.phase, w.wall, w.meta)
+
+
+def test_periodic_tank_with_a_piston(sphmod):
+    """Positions wrapped into the box and prescribed velocities, after steps and before the first."""
+    w = WL.wave_tank_small()
+    m = w.meta["piston"]
+    sim = sphmod.Simulation.from_workload(w)
+    sim.set_piston(m["axis"], m["amp"], m["omega"], m["phase"], m["t_end"])
+    _check(sim.diagnostics(), _state_of(sim, w))
+    sim.run(WL.stable_dt(w.params), 12)
+    _check(sim.diagnostics(), _state_of(sim, w))
+
+
+def test_instances_without_oil_among_others(sphmod):
+    ws = WL.drop_batch_2d(k=5, seed=79, d_range=(5.0, 14.0), perturb=True)
+    for q in (0, 3):
+        ws[q].phase[:] = 0
+    sim = sphmod.Simulation.batch(ws)
+    for _ in range(2):
+        for q, (d, w) in enumerate(zip(sim.diagnostics_instances(), ws)):
+            _check(d, w)
+            assert (d["n_oil"] == 0) == (q in (0, 3))
+            if q in (0, 3):
+                assert not np.any(d["centroid"])
+        sim.build_cells()
+
+
+@pytest.mark.parametrize("bad", ["nan", "-nan", "inf", "-inf"])
+def test_velocities_that_are_not_finite(sphmod, bad):
+    """The largest speed leaves out a NaN and keeps an infinity; sums over it are not finite, and
+    what does not read velocities is as it was."""
+    v = {"nan": np.nan, "-nan": -np.nan, "inf": np.inf, "-inf": -np.inf}[bad]
+    w = WL.drop_tank(2, (40, 44), drop_d_dx=12, seed=80, perturb=True)
+    at = np.flatnonzero(w.wall == 0)[717]
+    u = w.u.copy()
+    u[at, 1] = v
+    sim = sphmod.Simulation.from_workload(w)
+    ref = sim.diagnostics()
+    sim.set_state(w.x, u, w.rho)
+    d = sim.diagnostics()
+    others = np.delete(w.u, at, 0)[np.delete(w.wall, at) == 0]
+    if np.isnan(v):
+        assert d["u_max"] == np.sqrt((others ** 2).sum(1).max()) or \
+            abs(d["u_max"] / np.sqrt((others ** 2).sum(1).max()) - 1) < 1e-15
+        assert np.isnan(d["e_kin"]) and np.isnan(d["momentum"][1])
+    else:
+        assert d["u_max"] == np.inf and d["e_kin"] == np.inf and d["momentum"][1] == v
+    for k in ("mass", "e_pot", "sphericity", "n_oil"):
+        assert d[k] == ref[k], k
+    assert d["momentum"][0] == ref["momentum"][0] and np.array_equal(d["centroid"], ref["centroid"])
