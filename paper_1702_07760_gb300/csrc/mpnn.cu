@@ -341,12 +341,7 @@ __device__ __forceinline__ __half2 tanh_h2(__half2 x)
 // 1.05 -> 0.69 ms with 463 M warp instructions instead of 762 M, the FP16 half of
 // the FMA pipe 65 % busy.  Five blocks an SM (96 registers) and four edges in
 // flight measured best (jump 6.7 ms; six blocks 7.5, eight 7.3, eight edges 6.8).
-#ifndef EDGE_U
-#define EDGE_U 4
-#endif
-#ifndef EDGE_BLOCKS
-#define EDGE_BLOCKS 5
-#endif
+constexpr int EDGE_U = 4, EDGE_BLOCKS = 5;
 constexpr int EWF = 128;   // threads of the forward edge kernel (4 warps, two receivers each)
 
 template <int DIM>
@@ -735,8 +730,9 @@ __global__ void k_sums_out(const double *sum, float *grad, const __grid_constant
 }
 
 // Column sums over n rows of src (ld), optionally weighted per row, added to
-// dst: a thread per column and block of rows; the blocks' FP32 sums meet in FP64,
-// so the result does not depend on the order they finish in.
+// dst: a thread per column and block of rows; the blocks' FP32 sums meet in FP64
+// (atomics), so the order they finish in shows in the last bits of an FP64 sum only,
+// and after the rounding to FP32 in one unit of the last place at most.
 __global__ void k_colsum(const float *src, int ld, int cols, int n, const float *roww, double *dst)
 {
     const int c = threadIdx.x;
@@ -892,7 +888,6 @@ struct Epi {
     int act = 0;
     const float *dact = nullptr;
     int lddact = 0;
-    int cb_half = 0;
     // the P, Q layer: folded node terms (see umma::GemmArgs)
     const float4 *fold_f = nullptr;
     const float *fold_w = nullptr;
@@ -928,7 +923,6 @@ int mm(Surrogate &S, cudaStream_t st, const bf16 *A, int lda, const bf16 *B, int
     g.act = e.act;
     g.dact = e.dact;
     g.lddact = e.lddact;
-    g.cb_half = e.cb_half;
     g.err = S.err;
     if (e.fold_out) {
         g.fold_f = e.fold_f;
@@ -940,8 +934,9 @@ int mm(Surrogate &S, cudaStream_t st, const bf16 *A, int lda, const bf16 *B, int
         g.fold_out = e.fold_out;
         g.fold_ld = N;
     }
-    // every layer of the network has a shape of k_layer, whose epilogue alone folds and adds two residuals
-    cudaError_t err = umma::layer_fits(g) ? umma::layer(g, st) : cudaErrorInvalidValue;
+    // every layer of the network is k_layer's, which alone has its epilogues
+    const umma::LayerLaunch launch = umma::layer_for(g);
+    cudaError_t err = launch ? launch(g, st) : cudaErrorInvalidValue;
     if (err != cudaSuccess) return set_error(SPH_ECUDA, std::string("gemm: ") + cudaGetErrorString(err));
     return SPH_OK;
 }
@@ -1154,7 +1149,6 @@ int forward(Surrogate &S, const SimView &v, bool training)
             e.bias = S.bpq[r];
             // the backward pass reads the unfolded terms
             e.Cb = training ? (bf16 *)S.PQ[r] : nullptr;
-            e.cb_half = 1;
             e.ldcb = 2 * H;
             e.fold_f = S.NF;
             e.fold_w = T + L.w3[r];

@@ -12,13 +12,12 @@
 // copies: a chunk's arrival and the completion of its MMAs (tcgen05.commit)
 // are each signalled through an mbarrier; every wait gives up after one
 // second, raising an error flag, and the CTA waits (again bounded) for its
-// copies in flight and still releases its TMEM.  The epilogue reads the accumulator with tcgen05.ld
-// (each warp its 32-lane quarter), adds a column bias and an optional
-// row-scaled bias, stores the pre-activation, applies SiLU, adds a residual
-// and writes FP32 and/or BF16 (or FP16) outputs, or adds into FP32 with
+// copies in flight and still releases its TMEM.  The accumulator is read with tcgen05.ld
+// (each warp its 32-lane quarter) and stored as FP32, or added with
 // atomics when K is split across CTAs.  That is k_gemm, for any K and N; the
-// network's node layers run in k_layer (whole K in shared memory, persistent)
-// and its weight gradients in k_wgrad (operands as stored, no transposes).
+// network's node layers run in k_layer (whole K in shared memory, persistent,
+// with the layers' epilogues) and its weight gradients in k_wgrad (operands as
+// stored, no transposes).
 #pragma once
 
 #include <cuda.h>
@@ -219,7 +218,8 @@ struct GemmArgs {
     int k_split;                // K range of one CTA (multiple of 64); >= K: no split
     float *Cf;                  // FP32 output (or NULL)
     int ldcf;
-    __nv_bfloat16 *Cb;          // BF16 output (or NULL)
+    // from here to the fold for k_layer alone: k_gemm stores or adds the accumulator into Cf
+    __nv_bfloat16 *Cb;          // BF16 output (or NULL); FP16 (__half) with the fold
     int ldcb;
     const float *bias;          // per column (or NULL)
     const float *row_scale;     // C[r][c] += row_scale[r] * row_bias[c] (or NULL)
@@ -228,14 +228,12 @@ struct GemmArgs {
     int ldz;
     const float *residual;      // added after the activation (or NULL)
     int ldr;
-    const float *residual2;     // added to the residual first (or NULL; k_layer only)
+    const float *residual2;     // added to the residual first (or NULL)
     int ldr2;
     int act;                    // 0 none, 1 SiLU, 2 multiply by SiLU'(dact) (backward)
     const float *dact;          // pre-activation for act == 2
     int lddact;
-    int atomic;                 // 1: atomicAdd the raw accumulator into Cf (split K)
-    int n_store;                // columns stored (0: N)
-    int cb_half;                // 1: Cb holds FP16 (__half) instead of BF16
+    int atomic;                 // 1: atomicAdd the accumulator into Cf (k_gemm; split K)
     unsigned *err;              // error word (ERR_TIMEOUT)
     // k_layer<256, 128> only: the result [P | Q] (128 columns each, rounded to
     // FP16 as Cb holds it) with the linear form s = W3d . f of the row's node
@@ -249,72 +247,15 @@ struct GemmArgs {
 
 __device__ __forceinline__ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
-// 16 consecutive FP32 values: four 16-byte accesses when the chunk is whole
-// and aligned, else element by element (the first `count` values).
-__device__ __forceinline__ void store16(float *p, const float (&v)[16], bool full, int count)
+// 16 consecutive FP32 values: four 16-byte accesses when aligned, else element by element.
+__device__ __forceinline__ void store16(float *p, const float (&v)[16])
 {
-    if (full && aligned16(p)) {
+    if (aligned16(p)) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) ((float4 *)p)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     } else {
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if (j < count) p[j] = v[j];
-    }
-}
-
-__device__ __forceinline__ void load16(const float *p, float (&v)[16], bool full, int count)
-{
-    if (full && aligned16(p)) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 t = ((const float4 *)p)[q];
-            v[4 * q] = t.x;
-            v[4 * q + 1] = t.y;
-            v[4 * q + 2] = t.z;
-            v[4 * q + 3] = t.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = j < count ? p[j] : 0.f;
-    }
-}
-
-__device__ __forceinline__ void store16_half(__half *p, const float (&v)[16], bool full, int count)
-{
-    if (full && aligned16(p)) {
-        uint4 w[2];
-        uint32_t *u = (uint32_t *)w;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const __half2 b = __floats2half2_rn(v[2 * q], v[2 * q + 1]);
-            u[q] = *(const uint32_t *)&b;
-        }
-        ((uint4 *)p)[0] = w[0];
-        ((uint4 *)p)[1] = w[1];
-    } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if (j < count) p[j] = __float2half_rn(v[j]);
-    }
-}
-
-__device__ __forceinline__ void store16_bf16(__nv_bfloat16 *p, const float (&v)[16], bool full, int count)
-{
-    if (full && aligned16(p)) {
-        uint4 w[2];
-        uint32_t *u = (uint32_t *)w;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
-            u[q] = *(const uint32_t *)&b;
-        }
-        ((uint4 *)p)[0] = w[0];
-        ((uint4 *)p)[1] = w[1];
-    } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j)
-            if (j < count) p[j] = __float2bfloat16_rn(v[j]);
+        for (int j = 0; j < 16; ++j) p[j] = v[j];
     }
 }
 
@@ -446,47 +387,17 @@ __global__ void __launch_bounds__(THREADS, 1)
                     for (int j = 0; j < 16; ++j) v[j] = 0.f;
                 }
                 if (row >= g.M) continue;
-                const int nst = g.n_store > 0 ? g.n_store : BN;
-                // whole 16-column chunks go through 16-byte vector accesses
-                const bool full = c0 + 16 <= nst;
-                if (g.atomic) {
-                    float *dst = g.Cf + (size_t)row * g.ldcf + c0;
-                    if (full && aligned16(dst)) {
+                // 16-byte vector accesses where the row's address allows them
+                float *dst = g.Cf + (size_t)row * g.ldcf + c0;
+                if (!g.atomic) {
+                    store16(dst, v);
+                } else if (aligned16(dst)) {
 #pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            atomicAdd((float4 *)dst + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
-                    } else {
+                    for (int q = 0; q < 4; ++q)
+                        atomicAdd((float4 *)dst + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+                } else {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (c0 + j < nst) atomicAdd(dst + j, v[j]);
-                    }
-                    continue;
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    if (g.bias) v[j] += g.bias[c0 + j];
-                    if (g.row_scale) v[j] += g.row_scale[row] * g.row_bias[c0 + j];
-                }
-                if (g.Z) store16(g.Z + (size_t)row * g.ldz + c0, v, full, nst - c0);
-                if (g.act == 1) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = silu(v[j]);
-                } else if (g.act == 2) {
-                    float a[16];
-                    load16(g.dact + (size_t)row * g.lddact + c0, a, full, nst - c0);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] *= dsilu(a[j]);
-                }
-                if (g.residual) {
-                    float r[16];
-                    load16(g.residual + (size_t)row * g.ldr + c0, r, full, nst - c0);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] += r[j];
-                }
-                if (g.Cf) store16(g.Cf + (size_t)row * g.ldcf + c0, v, full, nst - c0);
-                if (g.Cb) {
-                    if (g.cb_half) store16_half((__half *)g.Cb + (size_t)row * g.ldcb + c0, v, full, nst - c0);
-                    else store16_bf16(g.Cb + (size_t)row * g.ldcb + c0, v, full, nst - c0);
+                    for (int j = 0; j < 16; ++j) atomicAdd(dst + j, v[j]);
                 }
             }
         }
@@ -918,24 +829,6 @@ inline bool make_map(CUtensorMap *m, const __nv_bfloat16 *base, int rows, int co
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Whether k_layer takes the contraction: the whole K in one tile (K and N as
-// the network's layers have them), every output row on 16-byte boundaries and
-// no split.  Everything else (other N or K, K split over blocks, odd leading
-// dimensions or addresses) is k_gemm's.
-inline bool layer_fits(const GemmArgs &g)
-{
-    const bool shape = (g.N == 128 && (g.K == 16 || g.K == 128 || g.K == 256)) || (g.N == 256 && g.K == 128) ||
-                       (g.N == 16 && g.K == 128);
-    auto ok = [](const void *p, int ld, int unit) { return !p || ((uintptr_t)p % 16 == 0 && ld % unit == 0); };
-    // one of activation, residual and fold; a pre-activation only with SiLU, FP16 only with the fold
-    const int kinds = (g.act != 0) + (g.residual != nullptr) + (g.fold_out != nullptr);
-    const bool epi = kinds <= 1 && (!g.Z || g.act == 1) && (!g.cb_half || g.fold_out) &&
-                     (!g.row_scale || kinds == 0);
-    return shape && epi && !g.atomic && g.k_split >= g.K && (g.n_store == 0 || g.n_store == g.N) && ok(g.Cf, g.ldcf, 4) &&
-           ok(g.Cb, g.ldcb, 4) && ok(g.Z, g.ldz, 4) && ok(g.residual, g.ldr, 4) && ok(g.residual2, g.ldr2, 4) &&
-           ok(g.dact, g.lddact, 4) && ok(g.bias, 0, 4) && ok(g.row_bias, 0, 4);
-}
-
 template <int BN, int K, int EPI>
 inline cudaError_t launch_layer(const GemmArgs &g, cudaStream_t stream)
 {
@@ -956,31 +849,42 @@ inline cudaError_t launch_layer(const GemmArgs &g, cudaStream_t stream)
     return cudaGetLastError();
 }
 
-// The epilogues each shape of the network is used with; cudaErrorInvalidValue for any other.
-inline cudaError_t layer(const GemmArgs &g, cudaStream_t stream)
+using LayerLaunch = cudaError_t (*)(const GemmArgs &, cudaStream_t);
+
+// The launch of the contraction by k_layer, NULL where it is not k_layer's.  The table holds the
+// shapes and epilogues of the network (and the plain product of each shape); besides, every
+// operand of the epilogue is on 16-byte boundaries in every row, and K is not split.  Plain and
+// accumulated products with other N or K, a split K, odd leading dimensions or addresses are
+// k_gemm's.
+inline LayerLaunch layer_for(const GemmArgs &g)
 {
+    auto ok = [](const void *p, int ld) { return !p || ((uintptr_t)p % 16 == 0 && ld % 4 == 0); };
+    if (g.atomic || g.k_split < g.K || !ok(g.Cf, g.ldcf) || !ok(g.Cb, g.ldcb) || !ok(g.Z, g.ldz) ||
+        !ok(g.residual, g.ldr) || !ok(g.residual2, g.ldr2) || !ok(g.dact, g.lddact) || !ok(g.bias, 0) ||
+        !ok(g.row_bias, 0))
+        return nullptr;
+    // one of activation, residual and fold; a pre-activation only with SiLU, a row-scaled bias with none
+    const int kinds = (g.act != 0) + (g.residual != nullptr) + (g.fold_out != nullptr);
+    if (kinds > 1 || (g.Z && g.act != 1) || (g.row_scale && kinds)) return nullptr;
     const int epi = g.fold_out ? EPI_FOLD
                                : (g.residual ? EPI_RESIDUAL : (g.act == 1 ? EPI_SILU : (g.act == 2 ? EPI_DSILU : EPI_PLAIN)));
-    const int id = (g.N * 1024 + g.K) * 8 + epi;
-#define SPH_LAYER_CASE(BN, K, EPI) \
-    case (BN * 1024 + K) * 8 + EPI: return launch_layer<BN, K, EPI>(g, stream);
-    switch (id) {
-        SPH_LAYER_CASE(128, 16, EPI_PLAIN)
-        SPH_LAYER_CASE(128, 16, EPI_SILU)
-        SPH_LAYER_CASE(128, 16, EPI_DSILU)
-        SPH_LAYER_CASE(128, 128, EPI_PLAIN)
-        SPH_LAYER_CASE(128, 128, EPI_SILU)
-        SPH_LAYER_CASE(128, 128, EPI_DSILU)
-        SPH_LAYER_CASE(128, 128, EPI_RESIDUAL)
-        SPH_LAYER_CASE(128, 256, EPI_PLAIN)
-        SPH_LAYER_CASE(128, 256, EPI_SILU)
-        SPH_LAYER_CASE(128, 256, EPI_RESIDUAL)
-        SPH_LAYER_CASE(256, 128, EPI_PLAIN)
-        SPH_LAYER_CASE(256, 128, EPI_FOLD)
-        SPH_LAYER_CASE(16, 128, EPI_PLAIN)
-    }
+#define SPH_LAYER_CASE(BN, KK, EPI) \
+    if (g.N == BN && g.K == KK && epi == EPI) return launch_layer<BN, KK, EPI>;
+    SPH_LAYER_CASE(128, 16, EPI_PLAIN)
+    SPH_LAYER_CASE(128, 16, EPI_SILU)
+    SPH_LAYER_CASE(128, 16, EPI_DSILU)
+    SPH_LAYER_CASE(128, 128, EPI_PLAIN)
+    SPH_LAYER_CASE(128, 128, EPI_SILU)
+    SPH_LAYER_CASE(128, 128, EPI_DSILU)
+    SPH_LAYER_CASE(128, 128, EPI_RESIDUAL)
+    SPH_LAYER_CASE(128, 256, EPI_PLAIN)
+    SPH_LAYER_CASE(128, 256, EPI_SILU)
+    SPH_LAYER_CASE(128, 256, EPI_RESIDUAL)
+    SPH_LAYER_CASE(256, 128, EPI_PLAIN)
+    SPH_LAYER_CASE(256, 128, EPI_FOLD)
+    SPH_LAYER_CASE(16, 128, EPI_PLAIN)
 #undef SPH_LAYER_CASE
-    return cudaErrorInvalidValue;
+    return nullptr;
 }
 
 // dW += dY^T X over n nodes: dY has fy features (rows of dW, 128 to a block
@@ -1015,13 +919,13 @@ inline cudaError_t wgrad(const __nv_bfloat16 *dY, int ldy, int fy, const __nv_bf
     return cudaGetLastError();
 }
 
-// Launches C = A B^T (+ epilogue) on `stream`; returns a cudaError_t.
+// Launches C = A B^T, stored in Cf or (atomic) added to it, on `stream`; returns a cudaError_t.
 inline cudaError_t gemm(const GemmArgs &g, cudaStream_t stream)
 {
     if (g.M <= 0) return cudaSuccess;
     if (g.K % 16 != 0 || g.lda % 8 != 0 || g.ldb % 8 != 0 || g.k_split % BK != 0 || g.k_split <= 0)
         return cudaErrorInvalidValue;
-    if (layer_fits(g)) return layer(g, stream);
+    if (const LayerLaunch l = layer_for(g)) return l(g, stream);
     const dim3 grid((g.M + BM - 1) / BM, (g.K + g.k_split - 1) / g.k_split);
     const size_t smem = gemm_smem_bytes(g.N);
     CUtensorMap mapA{}, mapB{};
