@@ -292,8 +292,9 @@ int sph_set_launch_shape(sph_handle h, int block, int grid_blocks, int dynamic_c
 int sph_get_launch_shape(sph_handle h, int *block, int *grid_blocks, int *dynamic_chunks);
 
 /* Times sph_run_persistent over trial_steps steps of size dt for every block
- * size in {128, 256, 512} with grids of every co-resident multiple of the SM
- * count, and, where the particles are fewer than twice such a grid's
+ * size in {128, 256, 512} with grids of every multiple of the SM count that is
+ * co-resident in the build grid_blocks = 0 takes (on inputs of at most 512
+ * particles per SM that is the one of 128 registers), and, where the particles are fewer than twice such a grid's
  * threads, of 1/2, 1/4, 1/8 and 1/19 of the SM count, each with both ways of
  * sharing out particles; keeps the fastest shape and writes it and its
  * milliseconds per step to the non-NULL outputs.
