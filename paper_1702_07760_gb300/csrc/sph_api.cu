@@ -1209,6 +1209,7 @@ int create_sim(const sph_params *params, int k, const int64_t *counts, const dou
              &s->rebuild_fit, dim == 2 ? (const void *)k_rebuild<2> : (const void *)k_rebuild<3>, 256, 0)) != cudaSuccess)
         return cuda_fail(e);
     s->rebuild_fit = std::min(s->rebuild_fit, 2);
+    a0.one_kernel = a1.one_kernel = s->rebuild_fit > 0 && n <= (int64_t)ONE_KERNEL_PER_SM * s->sms;
     {
         // super-cell centres per axis (the FP64 offsets' origins)
         std::vector<double> cen;

@@ -112,6 +112,7 @@ struct Grid {
 // All device arrays of one simulation (sorted order unless noted).
 struct Dev {
     int n;
+    int one_kernel;     // 1: a step's lists may be built by the one-kernel rebuild
     // state (FP64 accumulators + FP32 density deviation)
     double *x;          // dim * n, SoA
     double *u;          // dim * n, SoA
@@ -727,8 +728,9 @@ __device__ __forceinline__ void copy_one(const Dev &src, const Dev &dst, int k)
 
 // Whether a grid barrier of an earlier launch gave up: the lists may be unfinished, and
 // nothing is integrated until the host has reset the barrier.  (The lists that are there
-// hold valid indices at any time: empty ones from the creation on.)
-__device__ __forceinline__ bool stopped(const Dev &d) { return *d.flags & FLAG_TIMEOUT; }
+// hold valid indices at any time: empty ones from the creation on.)  Only inputs whose steps
+// may build in one kernel look at the flag.
+__device__ __forceinline__ bool stopped(const Dev &d) { return d.one_kernel && (*d.flags & FLAG_TIMEOUT); }
 
 // Neighbour list of particle i: every j != i within 2h + 2 skin at the
 // positions of the build, so the list stays complete while no particle moves
