@@ -72,3 +72,42 @@ def test_replayed_updates_take_their_own_step_size(env):  # noqa: F811
         expect, m, v = O.adam(theta, g, m, v, k + 1, lr)
         big = np.abs(g) > 1e-4 * np.abs(g).max()
         assert np.abs(sim.surrogate_weights() - expect)[big].max() < 2e-3 * lr
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_replays_between_steps_and_builds(env, dim):  # noqa: F811
+    """What moves the state, the lists and the handle's forms between two training steps: each
+    replay against the first step of a handle that has come the same way (a rates evaluation in
+    the place of each training step before, which builds the same lists)."""
+    from paper_1702_07760_gb300 import workloads as WL
+    torch, sph = env
+    w, norm, flat = _case(dim, 88 + dim)
+    dt = WL.stable_dt(w.params)
+
+    def timed(s):
+        s.timing(True)
+        s.run(dt, 3)
+        s.timing(False)
+
+    ways = [lambda s: None, lambda s: s.run(dt, 5), lambda s: s.run_persistent(dt, 3), lambda s: s.build_cells(),
+            lambda s: s.run(0.9 * dt, 9), timed, lambda s: s.set_state(*_state(w, 89)),
+            lambda s: (s.set_dt_scales([0.5]), s.run(dt, 2)), lambda s: s.set_launch_shape(128, 4)]
+    sim = sph.Simulation.from_workload(w)
+    sim.surrogate_init(flat, norm)
+    for k, way in enumerate(ways):
+        way(sim)
+        targets = _targets(torch, w, 110 + k)
+        t = [q.data_ptr() for q in targets]
+        loss, g = sim.surrogate_train_step(*t, update=False, want_grad=True)
+        one = sph.Simulation.from_workload(w)
+        for before in ways[:k]:
+            before(one)
+            one.eval_rates()
+        way(one)
+        one.surrogate_init(flat, norm)
+        loss1, g1 = one.surrogate_train_step(*t, update=False, want_grad=True)
+        assert abs(loss - loss1) <= 1e-10 * loss1, k
+        assert np.linalg.norm(g - g1) <= 1e-5 * np.linalg.norm(g1), k
+        for f in ("pos", "vel", "rho", "order"):
+            assert np.array_equal(sim.read(f), one.read(f)), (k, f)
+        one.close()
