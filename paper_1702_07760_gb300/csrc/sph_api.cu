@@ -115,8 +115,6 @@ PersistFn persist_fn(int dim, int bs, bool wide)
     return wide ? persist_fn_t<3, 512>(bs) : persist_fn_t<3, 1024>(bs);
 }
 
-}  // namespace
-
 // A driver function of the given version, looked up through the runtime; NULL when there is none.
 template <class F>
 F driver_fn(const char *name, int version)
@@ -144,6 +142,8 @@ cudaError_t stream_sms(cudaStream_t st, int *sms)
         *sms = std::min(*sms, (int)r.sm.smCount);
     return cudaSuccess;
 }
+
+}  // namespace
 
 struct sph_sim {
     sph_params P{};

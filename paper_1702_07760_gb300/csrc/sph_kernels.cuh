@@ -1692,10 +1692,10 @@ __device__ __forceinline__ unsigned rebuild_phases(const Dev &d, const Dev &scra
     for (int k = tid; k < n; k += stride) gather_one<DIM>(d, scratch, g, s, k);
     if ((f = grid_sync(bar, d.flags, state)) & stop) return f;
     if (tid == 0) *d.builds += 1;
-    // the copy apart from the list, which reads nothing it writes: in one loop the 2-D build of
-    // 128 registers reloaded 272 spilled bytes (4 drops of a batch, 20 steps 820 us; apart 792)
-    for (int k = tid; k < n; k += stride) copy_one<DIM>(scratch, d, k);
-    for_each_particle(bar, n, dyn, [&](int i) { list_one<DIM, false>(d, g, ph, scratch.tag, i); });
+    for_each_particle(bar, n, dyn, [&](int i) {
+        copy_one<DIM>(scratch, d, i);
+        list_one<DIM, false>(d, g, ph, scratch.tag, i);
+    });
     return f;
 }
 
