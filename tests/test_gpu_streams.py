@@ -99,3 +99,59 @@ def test_training_on_default_streams(env, dim, stream):  # noqa: F811
         loss1, g1 = ref.surrogate_train_step(*[a.data_ptr() for a in t], update=False, want_grad=True)
         assert abs(loss - loss1) <= 1e-10 * loss1
         assert np.linalg.norm(g - g1) <= 1e-5 * np.linalg.norm(g1)
+
+
+def test_handles_side_by_side(env):  # noqa: F811
+    """Several handles, each on its own stream and thread, whose cooperative rebuilds ask for the
+    whole device at the same time (75 k particles: 294 blocks of the 304 it holds), beside training
+    steps with streams of their own and a persistent run: the bits of each alone, and no time-out."""
+    import threading
+    torch, sph = env
+    tanks = [WL.drop_tank(2, (250, 288), drop_d_dx=70, seed=1, perturb=True),
+             WL.drop_tank(3, (34, 36, 40), drop_d_dx=10, seed=2, perturb=True),
+             WL.drop_tank(2, (120, 140), drop_d_dx=30, seed=3, perturb=True),
+             WL.drop_tank(2, (350, 380), drop_d_dx=80, seed=4, perturb=True)]
+
+    def steps(s, w, form):
+        dt = WL.stable_dt(w.params)
+        for k in range(40):
+            if form == "persistent":
+                s.run_persistent(dt, 10)
+            else:
+                s.run((1 - 0.01 * (k % 3)) * dt, 10, graph=form == "graph")
+            s.eval_rates()
+        return [s.read(f) for f in ("pos", "vel", "rho", "order", "acc")]
+
+    w, norm, flat = _case(2, 56)
+    t = [torch.tensor(a, dtype=torch.float64, device="cuda") for a in (w.x, w.u, w.rho)]
+    torch.cuda.synchronize()
+
+    def training(s):
+        s.surrogate_init(flat, norm)
+        return [s.surrogate_train_step(*[a.data_ptr() for a in t], update=False)[0] for _ in range(150)]
+
+    jobs = [(v, f) for v in tanks for f in ("graph", "eager")] + [(tanks[0], "persistent"), (tanks[2], "persistent")]
+    alone = [steps(sph.Simulation.from_workload(v), v, f) for v, f in jobs]
+    loss = training(sph.Simulation.from_workload(w))
+    sims = [sph.Simulation.from_workload(v) for v, _ in jobs]
+    trainer = sph.Simulation.from_workload(w)
+    got, failed = [None] * len(jobs), []
+
+    def work(q):
+        try:
+            if q < len(jobs):
+                got[q] = steps(sims[q], *jobs[q])
+            else:
+                assert np.allclose(training(trainer), loss, rtol=1e-10, atol=0)
+        except BaseException as e:  # noqa: BLE001 (reported below)
+            failed.append((q, e))
+
+    threads = [threading.Thread(target=work, args=(q,)) for q in range(len(jobs) + 1)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not failed, failed
+    for a, b in zip(alone, got):
+        for x, y in zip(a, b):
+            assert np.array_equal(x, y)
